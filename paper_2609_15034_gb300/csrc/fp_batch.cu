@@ -172,32 +172,21 @@ __device__ __forceinline__ void decode_queue(const BatchParams& bp, int q, u64 t
                                              unsigned char* area_raw, SlotSrc& rs) {
     typedef WarpCore<CODEC, K, false> C;
     const BatchQueue& Q = bp.q[q];
-    WarpArea<K>& area = *reinterpret_cast<WarpArea<K>*>(area_raw);
+    typename C::Area& area = *reinterpret_cast<typename C::Area*>(area_raw);
     const u32 lane = threadIdx.x & 31u;
     if (t >= t_end) return;
     // software pipeline as in the single-column decode: while tile t decodes,
-    // the inputs of t + W are in flight and the boundaries of t + 2W are read
+    // the inputs of t + W are in flight and the chunk of t + 2W is being read
     const SlotSrc* rc = Q.src + __ldg(Q.tile_chunk + t);
-    u32 lo, hi, lo1 = 0, hi1 = 0;
-    C::bounds(rc->p, t - rc->tile_base, lo, hi);
     typename C::Fetch cur;
-    C::fetch(rc->p, rc->x, bp.ex + rc->wt_base, t - rc->tile_base, lo, hi, cur);
-    const SlotSrc* rn = nullptr;
-    if (t + W < t_end) {
-        rn = Q.src + __ldg(Q.tile_chunk + t + W);
-        C::bounds(rn->p, t + W - rn->tile_base, lo1, hi1);
-    }
+    C::fetch(rc->p, rc->x, bp.ex + rc->wt_base, t - rc->tile_base, cur);
+    const SlotSrc* rn = t + W < t_end ? Q.src + __ldg(Q.tile_chunk + t + W) : nullptr;
     const SlotSrc* held = nullptr;   // the record copied into rs
     for (; t < t_end; t += W) {
         typename C::Fetch nxt;
         const u64 tn = t + W, t2 = t + 2 * W;
-        const SlotSrc* r2 = nullptr;
-        u32 lo2 = 0, hi2 = 0;
-        if (tn < t_end) C::fetch(rn->p, rn->x, bp.ex + rn->wt_base, tn - rn->tile_base, lo1, hi1, nxt);
-        if (t2 < t_end) {
-            r2 = Q.src + __ldg(Q.tile_chunk + t2);
-            C::bounds(r2->p, t2 - r2->tile_base, lo2, hi2);
-        }
+        if (tn < t_end) C::fetch(rn->p, rn->x, bp.ex + rn->wt_base, tn - rn->tile_base, nxt);
+        const SlotSrc* r2 = t2 < t_end ? Q.src + __ldg(Q.tile_chunk + t2) : nullptr;
         if (rc != held) {
             // the chunk's record into the warp's slot (the previous tile is done with it)
             const uint4* g = reinterpret_cast<const uint4*>(rc);
@@ -214,23 +203,23 @@ __device__ __forceinline__ void decode_queue(const BatchParams& bp, int q, u64 t
         cur = nxt;
         rc = rn;
         rn = r2;
-        lo1 = lo2;
-        hi1 = hi2;
     }
-    __syncwarp();   // the record slot is reused by the next queue
+    C::stage_free(lane);   // the area and the record slot are reused by the next queue
 }
 
-template <int K>
-struct WarpSlotBytes {
-    static constexpr size_t v = sizeof(WarpArea<K>);
+// Bytes of a warp's scratch area (one layout serves every codec's queue).
+template <int K16, int K12, int K8>
+struct WarpSlot {
+    static constexpr size_t a = sizeof(typename WarpCore<FP_ONPAIR16, K16, false>::Area);
+    static constexpr size_t b = sizeof(typename WarpCore<FP_ONPAIR12, K12, false>::Area);
+    static constexpr size_t c = sizeof(typename WarpCore<FP_FSST8, K8, false>::Area);
+    static constexpr size_t bytes = a > b ? (a > c ? a : c) : (b > c ? b : c);
 };
 
 template <int K16, int K12, int K8, int NW, int MINB>
 __global__ void __launch_bounds__(NW * 32, MINB) wbatch_decode_kernel(const BatchParams bp) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    constexpr size_t A = (WarpSlotBytes<K16>::v > WarpSlotBytes<K12>::v
-                              ? (WarpSlotBytes<K16>::v > WarpSlotBytes<K8>::v ? WarpSlotBytes<K16>::v : WarpSlotBytes<K8>::v)
-                              : (WarpSlotBytes<K12>::v > WarpSlotBytes<K8>::v ? WarpSlotBytes<K12>::v : WarpSlotBytes<K8>::v));
+    constexpr size_t A = WarpSlot<K16, K12, K8>::bytes;
     constexpr size_t SLOT = (A + sizeof(SlotSrc) + 15) / 16 * 16;
     static_assert(A % 16 == 0, "per-warp areas keep 16-byte alignment");
     const u32 warp = threadIdx.x >> 5;
@@ -248,12 +237,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) wbatch_decode_kernel(const Batc
 
 template <int K16, int K12, int K8, int NW>
 constexpr size_t wbatch_smem() {
-    return (size_t)NW * (((WarpSlotBytes<K16>::v > WarpSlotBytes<K12>::v
-                               ? (WarpSlotBytes<K16>::v > WarpSlotBytes<K8>::v ? WarpSlotBytes<K16>::v
-                                                                              : WarpSlotBytes<K8>::v)
-                               : (WarpSlotBytes<K12>::v > WarpSlotBytes<K8>::v ? WarpSlotBytes<K12>::v
-                                                                              : WarpSlotBytes<K8>::v)) +
-                          sizeof(SlotSrc) + 15) / 16 * 16);
+    return (size_t)NW * ((WarpSlot<K16, K12, K8>::bytes + sizeof(SlotSrc) + 15) / 16 * 16);
 }
 
 struct BatchKernel {

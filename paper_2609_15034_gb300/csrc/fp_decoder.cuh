@@ -440,27 +440,6 @@ struct Assembler {
         c[3] = fl ? s[7] : full.w;
         f &= 15u;   // below 16 before the insert, below 32 after it
     }
-    // Append a token of at most 8 bytes given already moved up by (f & 3)
-    // bytes (y0..y2, zero elsewhere): only whole-word moves remain, no
-    // funnel shifts.  Same stores and chunk handling as put().
-    __device__ __forceinline__ void put3(u32 y0, u32 y1, u32 y2, u32 len) {
-        const bool q1 = (f & 4u) != 0u;
-        const bool q2 = (f & 8u) != 0u;
-        const u32 v0 = q1 ? 0u : y0, v1 = q1 ? y0 : y1, v2 = q1 ? y1 : y2, v3 = q1 ? y2 : 0u;
-        const u32 s0 = q2 ? 0u : v0, s1 = q2 ? 0u : v1, s2 = q2 ? v0 : v2, s3 = q2 ? v1 : v3, s4 = q2 ? v2 : 0u,
-                  s5 = q2 ? v3 : 0u;
-        f += len;
-        const bool fl = f >= 16u;
-        const uint4 full = make_uint4(c[0] | s0, c[1] | s1, c[2] | s2, c[3] | s3);
-        if (fl) *tgt = full;
-        g += fl ? 1 : 0;
-        tgt = fl ? g : tgt;
-        c[0] = fl ? s4 : full.x;
-        c[1] = fl ? s5 : full.y;
-        c[2] = fl ? 0u : full.z;
-        c[3] = fl ? 0u : full.w;
-        f &= 15u;
-    }
     // Close the thread's range; `nonempty` = it produced at least one byte.
     // Afterwards the head slot holds the thread's lead fragment (FA_VALID).
     __device__ __forceinline__ void finish(bool nonempty) {
@@ -614,6 +593,21 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, u32 bytes, 
                  "l"(src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
 }
+
+// Copy `bytes` (a multiple of 16, both addresses 16-byte aligned) from shared
+// to global memory as a bulk group of the calling thread.
+__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, u32 bytes) {
+    asm volatile(
+        "cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\t"
+        "cp.async.bulk.commit_group;" ::"l"(dst),
+        "r"(smem_u32(src)), "r"(bytes)
+        : "memory");
+}
+// The calling thread's bulk copies have read their shared-memory source.
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// The calling thread's earlier shared-memory stores are visible to bulk
+// copies issued after a barrier that follows this.
+__device__ __forceinline__ void async_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // Bounded mbarrier waits give up after 4 s: well after any look-back has
 // given up (kSpinLimit), so a wait that a look-back holds up never expires

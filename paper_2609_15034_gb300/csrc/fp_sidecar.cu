@@ -87,16 +87,17 @@ template <int CODEC>
 struct Path {
     static constexpr int K = Shape<CODEC>::K;
     static constexpr bool DSMEM = Shape<CODEC>::DSMEM;
-    typedef WarpCore<CODEC, K, DSMEM> C;
+    // dictionary reads: whole 16-byte entries for the OnPair codecs (staged
+    // for OnPair-12, through L1 for OnPair-16), 8-byte entries for FSST; the
+    // length table staged for all
+    static constexpr int W = (CODEC == FP_ONPAIR16 || CODEC == FP_ONPAIR12) ? 16 : 8;
+    typedef WarpCore<CODEC, K, DSMEM, W, false, true> C;
 
     static size_t decode_smem() {
-        return (size_t)C::DICT_BYTES + (DSMEM ? (size_t)C::LENS_BYTES : 0) + kSidecarWarps * sizeof(WarpArea<K>);
+        return (size_t)C::STAGED_BYTES + kSidecarWarps * sizeof(typename C::Area);
     }
-    // dictionary reads: whole 16-byte entries for the OnPair codecs (staged
-    // for OnPair-12, through L1 for OnPair-16), 8-byte entries for FSST
-    static constexpr int W = (CODEC == FP_ONPAIR16 || CODEC == FP_ONPAIR12) ? 16 : 8;
     static const void* decode_kernel() {
-        return (const void*)&warp_decode_kernel<CODEC, K, DSMEM, kSidecarWarps, 1, W>;
+        return (const void*)&warp_decode_kernel<CODEC, K, DSMEM, kSidecarWarps, 1, W, false, true>;
     }
     // Index pass in blocks [0, ib), reduce in the next rg blocks (rg = 0: index only).
     static cudaError_t index_reduce(const DecodeParams& p, Extent* xp, u64* agg, uint64_t ib, uint64_t rg,

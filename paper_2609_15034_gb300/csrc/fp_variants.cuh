@@ -28,15 +28,15 @@ Variant make_variant() {
     return v;
 }
 
-template <int CODEC, int K, bool DSMEM, int NW, int MINB, int W>
+template <int CODEC, int K, bool DSMEM, int NW, int MINB, int W, bool LSMEM = DSMEM>
 Variant make_warp_variant() {
-    typedef WarpCore<CODEC, K, DSMEM, W> C;
+    typedef WarpCore<CODEC, K, DSMEM, W, false, LSMEM> C;
     Variant v{};
     v.threads = NW * 32;
     v.slots_per_thread = K;
     v.dict_smem = DSMEM ? 1 : 0;
-    v.smem_bytes = (size_t)C::DICT_BYTES + (DSMEM ? (size_t)C::LENS_BYTES : 0) + NW * sizeof(WarpArea<K>);
-    v.kernel = (const void*)&warp_decode_kernel<CODEC, K, DSMEM, NW, MINB, W>;
+    v.smem_bytes = (size_t)C::STAGED_BYTES + NW * sizeof(typename C::Area);
+    v.kernel = (const void*)&warp_decode_kernel<CODEC, K, DSMEM, NW, MINB, W, false, LSMEM>;
     v.warp_tiles = 1;
     v.reduce = (const void*)&reduce_kernel<CODEC, K, DSMEM>;
     v.scan = (const void*)&tiles_scan_kernel<CODEC == FP_FSST8>;
@@ -52,7 +52,7 @@ Variant make_fused_variant() {
     v.threads = NW * 32;
     v.slots_per_thread = K;
     v.dict_smem = DSMEM ? 1 : 0;
-    v.smem_bytes = (size_t)C::DICT_BYTES + (DSMEM ? (size_t)C::LENS_BYTES : 0) + NW * sizeof(WarpArea<K>);
+    v.smem_bytes = (size_t)C::STAGED_BYTES + NW * sizeof(typename C::Area);
     v.kernel = (const void*)&fused_decode_kernel<CODEC, K, DSMEM, NW, W>;
     v.warp_tiles = 2;
     v.width = W;
@@ -64,14 +64,14 @@ Variant make_fused_variant() {
 template <int CODEC, bool DSMEM, int NW>
 Variant make_packed_variant() {
     constexpr int K = 16, W = (CODEC == FP_FSST12) ? 8 : 16;
-    typedef WarpCore<CODEC, K, DSMEM, W, true> C;
+    typedef WarpCore<CODEC, K, DSMEM, W, true, true> C;
     Variant v{};
     v.threads = NW * 32;
     v.slots_per_thread = K;
     v.dict_smem = DSMEM ? 1 : 0;
-    v.smem_bytes = (size_t)C::DICT_BYTES + (DSMEM ? (size_t)C::LENS_BYTES : 0) + NW * sizeof(WarpArea<K>) +
+    v.smem_bytes = (size_t)C::STAGED_BYTES + NW * sizeof(typename C::Area) +
                    (size_t)NW * 32 * C::PK_STRIDE * sizeof(u32);
-    v.kernel = (const void*)&warp_decode_kernel<CODEC, K, DSMEM, NW, 1, W, true>;
+    v.kernel = (const void*)&warp_decode_kernel<CODEC, K, DSMEM, NW, 1, W, true, true>;
     v.warp_tiles = 1;
     v.reduce = (const void*)&reduce_kernel<CODEC, K, DSMEM, true>;
     v.scan = (const void*)&tiles_scan_kernel<false>;

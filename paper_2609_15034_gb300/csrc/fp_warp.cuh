@@ -13,17 +13,18 @@
 //                   escape state;
 //   warp_decode_kernel  every warp decodes whole warp tiles on its own: code
 //                   unpack, lengths, a warp scan inside the tile, assembly in
-//                   registers with aligned 16-byte stores, merging of chunks
-//                   shared by lanes through a per-warp shared-memory area,
-//                   string offsets.  No block barrier and no wait on other
-//                   warps, so the SM hides the latency of one warp's loads with
-//                   the others' work.
+//                   a per-warp staging area in shared memory, one bulk copy
+//                   of its whole 16-byte chunks, string offsets.  No block
+//                   barrier and no wait on other warps, so the SM hides the
+//                   latency of one warp's loads with the others' work.
 //
 // Reading the code stream twice costs its bytes (about a fifth of the
 // traffic at 6 decoded bytes per 12-bit code) but removes the serial
 // look-back from the decode itself; this is the paper's sidecar (Sec. 3.1)
 // regenerated on the device by the first two passes.
 #pragma once
+#include <type_traits>
+
 #include "fp_decoder.cuh"
 
 namespace fp {
@@ -41,63 +42,83 @@ __device__ __forceinline__ Elem wt_unpack(u64 w) {
     return Elem{w & 0xffffffull, (w >> 24) & 0xffffffull, (u32)((w >> 48) & 3u)};
 }
 
-// A chunk of which only bytes [lo, hi) may be written (shared with a
-// neighbouring warp tile).
-struct Partial {
-    uint4 v;
-    uint4* chunk;
-    u32 lo, hi;
-    bool pending;
+// A read-only load that stays where it is written (the compiler may move
+// __ldg() down to its use, behind the work that should hide it).
+__device__ __forceinline__ u32 ld_here(const u32* a) {
+    u32 v;
+    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(a));
+    return v;
+}
+
+// A lane's run of tokens appended to the warp's staging area as aligned
+// 32-bit words: `m` bytes of the current word (at `at`) are in `c`.
+//
+// Words in shared memory instead of 16-byte chunks in registers: moving a
+// token to a byte offset inside a word takes five funnel shifts and four
+// selects, moving it inside a 16-byte window took about 12 selects and 8
+// funnel shifts, and that integer work bound the decode (ALU pipe 64-72 %
+// active).  OnPair-12, 36M codes: 85 -> 65 instructions per code, the decode
+// kernel 149 -> 118 us; FSST-8, 38M slots: 77 -> 54, 134 -> 100 us.  What
+// bounds it now is the shared-memory pipe (79 % of its wavefronts on
+// OnPair-12): about 10 wavefronts per 32 codes for the table reads, 10 for
+// these stores, 3 for the lengths.
+struct StageWriter {
+    u32* at;
+    u32 m, c;
+
+    // Continue at staging byte `pos`; a word begun by the lanes before is
+    // completed here with their bytes zero, and they add theirs by
+    // finish().
+    __device__ __forceinline__ void begin(u32* stage, u32 pos) {
+        at = stage + (pos >> 2);
+        m = pos & 3u;
+        c = 0u;
+    }
+    // Append a token of up to 16 bytes (zero past its length).
+    __device__ __forceinline__ void put(const uint4 t, u32 len) {
+        const u32 sh = m * 8u;
+        const u32 s0 = c | __funnelshift_l(0u, t.x, sh), s1 = __funnelshift_l(t.x, t.y, sh),
+                  s2 = __funnelshift_l(t.y, t.z, sh), s3 = __funnelshift_l(t.z, t.w, sh),
+                  s4 = __funnelshift_l(t.w, 0u, sh);
+        const u32 e = m + len;
+        if (e >= 4u) at[0] = s0;
+        if (e >= 8u) at[1] = s1;
+        if (e >= 12u) at[2] = s2;
+        if (e >= 16u) at[3] = s3;
+        c = e >= 4u ? s1 : s0;
+        c = e >= 8u ? s2 : c;
+        c = e >= 12u ? s3 : c;
+        c = e >= 16u ? s4 : c;
+        at += e >> 2;
+        m = e & 3u;
+    }
+    // Append a token of up to 8 bytes (zero past its length).
+    __device__ __forceinline__ void put8(const uint2 t, u32 len) {
+        const u32 sh = m * 8u;
+        const u32 s0 = c | __funnelshift_l(0u, t.x, sh), s1 = __funnelshift_l(t.x, t.y, sh),
+                  s2 = __funnelshift_l(t.y, 0u, sh);
+        const u32 e = m + len;
+        if (e >= 4u) at[0] = s0;
+        if (e >= 8u) at[1] = s1;
+        c = e >= 4u ? s1 : s0;
+        c = e >= 8u ? s2 : c;
+        at += e >> 2;
+        m = e & 3u;
+    }
+    // The lane's bytes of a word that a following lane completed (every lane
+    // of the warp has stored its words).
+    __device__ __forceinline__ void finish() {
+        if (c) atomicOr(at, c);
+    }
 };
 
-// Merge a partial chunk with the lead fragments of the following lanes of
-// the same warp tile; store it if it is complete, else leave it pending for
-// store_partials().
-__device__ __forceinline__ void combine_lanes(uint4* chunk, uint4 acc, u32 lo, u32 hi, int m, const uint4* s_fa,
-                                              const u32* s_meta, Partial& pend) {
-    while (hi < 16u && m < 32) {
-        const u32 mm = s_meta[m];
-        if (mm & FA_VALID) {
-            acc = or4(acc, s_fa[m]);
-            hi = (mm >> FA_HI_SHIFT) & 31u;
-        }
-        ++m;
-    }
-    if (lo == 0u && hi == 16u) {
-        __stcs(chunk, acc);
-    } else {
-        pend.v = acc;
-        pend.chunk = chunk;
-        pend.lo = lo;
-        pend.hi = hi;
-        pend.pending = true;
-    }
-}
-
-// The warp writes its lanes' pending partial chunks together: lane b stores
-// byte b of a chunk when b is in [lo, hi), one byte store per chunk.
-__device__ __forceinline__ void store_partials(const Partial& pd) {
-    const u32 lane = threadIdx.x & 31u;
-    u32 ball = __ballot_sync(0xffffffffu, pd.pending);
-    while (ball) {
-        const int src = __ffs(ball) - 1;
-        ball &= ball - 1u;
-        const u32 x = __shfl_sync(0xffffffffu, pd.v.x, src), y = __shfl_sync(0xffffffffu, pd.v.y, src);
-        const u32 z = __shfl_sync(0xffffffffu, pd.v.z, src), w = __shfl_sync(0xffffffffu, pd.v.w, src);
-        const u32 lo = __shfl_sync(0xffffffffu, pd.lo, src), hi = __shfl_sync(0xffffffffu, pd.hi, src);
-        const unsigned long long a = __shfl_sync(0xffffffffu, (unsigned long long)pd.chunk, src);
-        const u32 q = lane >> 2;
-        const u32 word = q == 0 ? x : (q == 1 ? y : (q == 2 ? z : w));
-        if (lane >= lo && lane < hi) reinterpret_cast<uint8_t*>(a)[lane] = (uint8_t)(word >> ((lane & 3u) * 8u));
-    }
-}
-
-// Per-warp shared-memory area of the decode kernel.
-template <int K>
+// Per-warp shared-memory area of the decode kernel.  `stage` holds up to CAP
+// decoded bytes, at the alignment they have in the output, so that the whole
+// 16-byte chunks leave by one bulk copy per tile (no store instructions, and
+// no scattered lines in L1).
+template <int K, int CAP>
 struct WarpArea {
-    uint4 fa[32];
-    uint4 fb[32];
-    u32 meta[32];
+    uint4 stage[CAP / 16 + 1];
     u32 pre[K / 4][32];     // tile-relative output offset of slot 4m of each lane
     u32 contrib[K / 4][32]; // bytes each slot produced, one byte per slot
     u32 lit_mask[32];       // FSST-8: bit k = slot k holds a literal byte
@@ -110,8 +131,12 @@ struct WarpArea {
 // PACKED: the codes are stored bit-packed at p.packed_bits bits per code
 // (LSB-first, 1..16) instead of the codec's own layout -- the cascade layer
 // the paper removes on the host (Sec. 5), unpacked here inside the kernels.
+// LSMEM: the length table is staged in shared memory (with DSMEM the
+// dictionary too).  OnPair-16 stages its 64 KiB of lengths: a gather of 32
+// bytes takes about 3 wavefronts there against 10 through L1, whose lines
+// then serve the tokens (40M codes: 250 -> 210 us per call).
 template <int CODEC, int K, bool DSMEM, int W = (CODEC == FP_ONPAIR16 || CODEC == FP_ONPAIR12) ? 16 : 8,
-          bool PACKED = false>
+          bool PACKED = false, bool LSMEM = DSMEM>
 struct WarpCore {
     static constexpr bool FSST = (CODEC == FP_FSST8);   // escape codec: two-state scan elements
     static constexpr bool TOK8 = (CODEC == FP_FSST8 || CODEC == FP_FSST12);   // 8-byte table entries
@@ -128,13 +153,17 @@ struct WarpCore {
     static constexpr int PK_STRIDE = 2 * LANE_WORDS;
     // entries of the table (a staged table, or the global planes)
     static constexpr int kTable = (CODEC == FP_FSST8) ? 256 : (CODEC == FP_ONPAIR16 ? 65536 : 4096);
-    // FSST-8 with a staged table: every symbol and every literal byte kept
-    // moved up by 0..3 bytes (entry lit * 1024 + r * 256 + b, 16 bytes
-    // each), so an insert at byte position f reads the copy for r = f & 3
-    // and needs only whole-word moves.
-    static constexpr bool PRESHIFT = FSST && DSMEM;
-    static constexpr int DICT_BYTES = DSMEM ? (PRESHIFT ? 2 * 4 * 256 * 16 : kTable * (TOK8 ? 8 : 16)) : 0;
-    static constexpr int LENS_BYTES = kTable;
+    // FSST-8 with a staged table: the symbols, then the 256 literal bytes as
+    // tokens of their own, so a slot reads entry code + 256 * literal.
+    static constexpr bool LITTAB = FSST && DSMEM;
+    static constexpr int DICT_BYTES = DSMEM ? (kTable + (LITTAB ? 256 : 0)) * (TOK8 ? 8 : 16) : 0;
+    // Staged output bytes of a warp: an ordinary tile in one round (512
+    // tokens of 7.5 bytes: 3.8 KB; 1,024 FSST symbols: 4.6 KB); less where
+    // the dictionary is read through L1, which shares the SM's memory.
+    static constexpr int CAP = DSMEM ? 6144 : 4096;
+    typedef WarpArea<K, CAP> Area;
+    static constexpr int LENS_BYTES = LSMEM ? kTable : 0;
+    static constexpr int STAGED_BYTES = DICT_BYTES + LENS_BYTES;   // tables in front of the warp areas
     typedef TileRegs<CODEC, K> R;
     static_assert(K == 8 || K == 16 || K == 32, "slots per lane");
     static_assert(!FSST || K >= 16, "FSST-8 handles 16 slots at a time");
@@ -308,7 +337,7 @@ struct WarpCore {
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
                 const u32 code = code_at<CODEC, K>(r, 4 * j + h);
-                const u32 L = DSMEM ? (u32)lens[code] : (u32)__ldg(lens + code);
+                const u32 L = LSMEM ? (u32)lens[code] : (u32)__ldg(lens + code);
                 w |= L << (8 * h);
             }
             r.L[j] = w;
@@ -448,80 +477,98 @@ struct WarpCore {
         return make_uint4(a.x, a.y, b.x, b.y);
     }
 
+    // Token of an FSST slot, zero past its length.  FSST-8: a literal's byte,
+    // else the symbol; a slot that yields no byte is an escape or a corrupt
+    // code, whose table entries (255, and those past the dictionary) are all
+    // zero, so in a lane whose slots are all inside the column only literals
+    // need a select.
+    static __device__ __forceinline__ uint2 token8(const DecodeParams& p, const uint4* dict, u32 code, bool lit) {
+        const uint2* tab = DSMEM ? reinterpret_cast<const uint2*>(dict) : reinterpret_cast<const uint2*>(p.dict.table);
+        if (LITTAB) return tab[code | (lit ? 256u : 0u)];
+        const uint2 d = DSMEM ? tab[code] : __ldg(tab + code);
+        return (FSST && lit) ? make_uint2(code, 0u) : d;
+    }
+
+    // Append the lane's K tokens (cw: the bytes of each slot, `lit` its
+    // literals) in two independent runs, slots 0 .. K/2 - 1 by w0 and the
+    // others by w1: an append waits for the one before it in its run, so two
+    // runs hide half of that wait.  The next four tokens are read while four
+    // are appended: the compiler cannot move dictionary reads over the
+    // staging stores itself.
     template <bool ALLV>
-    static __device__ __forceinline__ void assemble_onpair(const DecodeParams& p, const uint4* dict, const R& r,
-                                                           Assembler& as) {
-#pragma unroll
-        for (int k0 = 0; k0 < K; k0 += 4) {
-            uint4 tok[4];
-#pragma unroll
-            for (int h = 0; h < 4; ++h)
-                tok[h] = token(p, dict, code_at<CODEC, K>(r, k0 + h), len_at<CODEC, K>(r, k0 + h));
+    static __device__ __forceinline__ void assemble(const DecodeParams& p, const uint4* dict, const R& r,
+                                                    const u32 (&cw)[K / 4], u32 lit, StageWriter& w0,
+                                                    StageWriter& w1) {
+        typedef typename std::conditional<TOK8, uint2, uint4>::type Tok;
+        Tok tok[2][4];
+        // step g: slots 2g, 2g + 1 and K/2 + 2g, K/2 + 2g + 1
+        auto slot = [](int g, int h) { return 2 * g + (h & 1) + (h >> 1) * (K / 2); };
+        auto bytes = [&](int k) { return (cw[k >> 2] >> (8 * (k & 3))) & 0xffu; };
+        auto load = [&](int g) {
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
-                const int k = k0 + h;
-                if (ALLV) {
-                    as.put(tok[h], len_at<CODEC, K>(r, k));
+                const int k = slot(g, h);
+                const u32 code = code_at<CODEC, K>(r, k);
+                Tok& t = tok[g & 1][h];
+                if constexpr (TOK8) t = token8(p, dict, code, (lit >> k) & 1u);
+                else t = token(p, dict, code, len_at<CODEC, K>(r, k));
+                if (!ALLV && bytes(k) == 0u) t = Tok{};
+            }
+        };
+        load(0);
+#pragma unroll
+        for (int g = 0; g < K / 4; ++g) {
+            if (g + 1 < K / 4) load(g + 1);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if constexpr (TOK8) {
+                    w0.put8(tok[g & 1][h], bytes(slot(g, h)));
+                    w1.put8(tok[g & 1][h + 2], bytes(slot(g, h + 2)));
                 } else {
-                    const bool v = (r.valid >> k) & 1u;
-                    as.put(v ? tok[h] : make_uint4(0, 0, 0, 0), v ? len_at<CODEC, K>(r, k) : 0u);
+                    w0.put(tok[g & 1][h], bytes(slot(g, h)));
+                    w1.put(tok[g & 1][h + 2], bytes(slot(g, h + 2)));
                 }
             }
         }
     }
 
-    // FSST-8 slots: a literal's byte, else the symbol; cw holds each slot's
-    // byte count.  In a lane whose slots are all inside the column a slot
-    // that yields no byte is an escape or a corrupt code, whose table entries
-    // (255, and those past the dictionary) are all zero, so only literals
-    // need a select there.
-    template <bool ALLV>
-    static __device__ __forceinline__ void assemble_fsst(const DecodeParams& p, const uint4* dict, const R& r,
-                                                         const u32 (&cw)[K / 4], u32 lit, Assembler& as) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const u32 bt = code_at<CODEC, K>(r, k);
-            const u32 a = (cw[k >> 2] >> ((k & 3) * 8)) & 0xffu;
-            const bool is_lit = (lit >> k) & 1u;
-            if (PRESHIFT) {
-                // the copy of the symbol (or literal) moved up by the insert position's byte offset
-                uint4 y = dict[(((lit >> k) & 1u) << 10) | ((as.f & 3u) << 8) | bt];
-                if (!ALLV && a == 0u) y = make_uint4(0u, 0u, 0u, 0u);
-                as.put3(y.x, y.y, y.z, a);
-                continue;
-            }
-            uint2 d;
-            if (DSMEM) d = reinterpret_cast<const uint2*>(dict)[bt];
-            else d = __ldg(reinterpret_cast<const uint2*>(p.dict.table) + bt);
-            uint4 tok;
-            if (ALLV) tok = make_uint4(is_lit ? bt : d.x, is_lit ? 0u : d.y, 0u, 0u);
-            else tok = make_uint4(a == 0u ? 0u : (is_lit ? bt : d.x), (a == 0u || is_lit) ? 0u : d.y, 0u, 0u);
-            as.put(tok, a);
+    // Write the staged bytes [off0, nb) to the 16-byte chunks from g on:
+    // the whole chunks by one bulk copy (left in flight: stage_free() before
+    // the area is written again), the bytes of the two edge chunks, shared
+    // with the neighbouring tiles, one per lane.  Every lane has fenced its
+    // stores for the copy engine.
+    static __device__ __forceinline__ void flush(const uint4* stage, uint4* g, u32 off0, u32 nb, u32 lane) {
+        const u32 first = off0 ? 1u : 0u, last = nb >> 4;
+        if (lane == 0u && last > first) bulk_s2g(g + first, stage + first, (last - first) * 16u);
+        const u32 b = lane & 15u, e = nb & 15u;
+        const bool head = lane < 16u;
+        const bool w = head ? (off0 != 0u && b >= off0 && b < nb) : (b < e && !(last == 0u && off0 != 0u));
+        if (w) {
+            const u32 i = head ? b : last * 16u + b;
+            reinterpret_cast<uint8_t*>(g)[i] = reinterpret_cast<const uint8_t*>(stage)[i];
         }
+    }
+    // The copy engine has read what the last flush() gave it (every lane of
+    // the warp calls this).
+    static __device__ __forceinline__ void stage_free(u32 lane) {
+        if (lane == 0u) bulk_wait_read();
+        __syncwarp();
     }
 
     // Stage the dictionary and the token lengths in shared memory (every
     // thread of the block; the caller synchronises).  FSST: the 8-byte
-    // entries, or for FSST-8 the moved-up copies (PRESHIFT); OnPair read
+    // entries, for FSST-8 with the literals after them (LITTAB); OnPair read
     // whole (W = 16): the 16-byte entries; OnPair split read (W = 8): the two
     // planes (entry e's bytes 0..7 at low-plane word e, bytes 8..15 at
     // high-plane word e).
     static __device__ __forceinline__ void stage_dict(const DecodeParams& p, uint4* s_dict, uint8_t* s_lens,
                                                       int nthreads) {
-        if (!DSMEM) return;
-        if (PRESHIFT) {
+        if (!LSMEM) return;
+        if (LITTAB) {
             const uint2* tab = reinterpret_cast<const uint2*>(p.dict.table);
-            for (int i = threadIdx.x; i < DICT_BYTES / 16; i += nthreads) {
-                const u32 b = (u32)i & 255u, r8 = (((u32)i >> 8) & 3u) * 8u;
-                u32 lo = b, hi = 0u;   // a literal byte
-                if (i < 1024) {
-                    const uint2 d = __ldg(tab + b);
-                    lo = d.x;
-                    hi = d.y;
-                }
-                s_dict[i] = make_uint4(lo << r8, __funnelshift_l(lo, hi, r8), __funnelshift_l(hi, 0u, r8), 0u);
-            }
-        } else {
+            for (int i = threadIdx.x; i < 512; i += nthreads)
+                reinterpret_cast<uint2*>(s_dict)[i] = i < 256 ? __ldg(tab + i) : make_uint2((u32)i - 256u, 0u);
+        } else if (DSMEM) {
             const uint4* src = reinterpret_cast<const uint4*>((TOK8 || W == 16) ? p.dict.table : p.dict.planes);
             for (int i = threadIdx.x; i < DICT_BYTES / 16; i += nthreads) s_dict[i] = __ldg(src + i);
         }
@@ -530,12 +577,12 @@ struct WarpCore {
     }
 
     // The same staging by the bulk-copy engine where the staged layout is the
-    // stored one (no planes, no moved-up copies): thread 0 issues the two
+    // stored one (no planes, no literals): thread 0 issues the two
     // copies (cp.async.bulk, completion counted on one mbarrier) and every
     // thread waits for them, bounded (a wait that gives up sets
     // ERRB_TIMEOUT).  Falls back to the loads above for tables that are not
     // 16-byte aligned.  Every thread of the block calls it; returns synchronised.
-    static constexpr bool BULK_STAGE = DSMEM && !PRESHIFT && (TOK8 || W == 16);
+    static constexpr bool BULK_STAGE = LSMEM && !LITTAB && (!DSMEM || TOK8 || W == 16);
     static __device__ __forceinline__ void stage_dict_bulk(const DecodeParams& p, uint4* s_dict, uint8_t* s_lens,
                                                            u64* bar, int nthreads) {
         const bool aligned =
@@ -549,7 +596,7 @@ struct WarpCore {
             mbar_init(bar, 1u);
             mbar_init_fence();
             mbar_expect_tx(bar, (u32)(DICT_BYTES + LENS_BYTES));
-            bulk_g2s(s_dict, p.dict.table, (u32)DICT_BYTES, bar);
+            if (DSMEM) bulk_g2s(s_dict, p.dict.table, (u32)DICT_BYTES, bar);
             bulk_g2s(s_lens, p.dict.lens, (u32)LENS_BYTES, bar);
             mbar_arrive(bar);
         }
@@ -570,7 +617,7 @@ struct WarpCore {
         for (int k = 0; k < K; ++k) {
             const int bit = k * WBITS, w = bit >> 5, sh = bit & 31;
             const u32 code = (sh + WBITS <= 32) ? ((wv[w] >> sh) & MASK) : (__funnelshift_r(wv[w], wv[w + 1], sh) & MASK);
-            const u32 L = DSMEM ? (u32)lens[code] : (u32)__ldg(lens + code);
+            const u32 L = LSMEM ? (u32)lens[code] : (u32)__ldg(lens + code);
             sum += L;
             mn = min(mn, L);
         }
@@ -583,47 +630,30 @@ struct WarpCore {
     }
 
     // Inputs of a warp tile fetched ahead of its decode: the lane's code
-    // words, the tile's scanned offset, its string boundaries [lo, hi) and
-    // the first PB*32 of their code_offsets (one per lane and round).
-    static constexpr int PB = FSST ? 2 : 1;
+    // words, the tile's scanned offset, its string boundaries [lo, hi) (as
+    // stored: clamped where they are used, so that nothing waits for the
+    // loads here).
     struct Fetch {
         u32 wv[LANE_WORDS];
         bool fast;
         u64 ex;
         u32 lo, hi;
-        u32 pos[PB];
     };
+    // Rounds of 32 boundaries whose code_offsets are in flight together.
+    static constexpr int PB = K / 8;
 
     // Loads of data written by this launch's earlier phases (the one-launch
     // decode, CG) bypass L1; otherwise the read-only path.
     template <bool CG, class T>
     static __device__ __forceinline__ T ld(const T* a) { return CG ? __ldcg(a) : __ldg(a); }
 
-    // Issue the loads of tile t whose boundaries [lo, hi) are already known.
+    // Issue the loads of tile t.
     template <bool CG = false>
-    static __device__ __forceinline__ void fetch(const DecodeParams& p, const Extent& x, const u64* ex, u64 t, u32 lo,
-                                                 u32 hi, Fetch& f) {
-        const u32 lane = threadIdx.x & 31u;
+    static __device__ __forceinline__ void fetch(const DecodeParams& p, const Extent& x, const u64* ex, u64 t, Fetch& f) {
         f.fast = load_fast(p, lane_q0(x, t), f.wv);
         f.ex = ld<CG>(ex + t);
-        f.lo = lo;
-        f.hi = hi;
-#pragma unroll
-        for (int j = 0; j < PB; ++j) {
-            const u32 i = lo + lane + 32u * j;
-            f.pos[j] = i < hi ? __ldg(p.code_offsets + i) : 0u;
-        }
-    }
-
-    // Boundaries [lo, hi) of tile t, clamped to the column's.
-    template <bool CG = false>
-    static __device__ __forceinline__ void bounds(const DecodeParams& p, u64 t, u32& lo, u32& hi) {
-        const u64 nb = (u64)p.n_strings + 1;
-        lo = ld<CG>(p.first + t);
-        hi = ld<CG>(p.first + t + 1);
-        if ((u64)lo > nb) lo = (u32)nb;
-        if ((u64)hi > nb) hi = (u32)nb;
-        if (hi < lo) hi = lo;
+        f.lo = ld<CG>(p.first + t);
+        f.hi = ld<CG>(p.first + t + 1);
     }
 
     // Decode warp tile t of column (p, x) from its fetched inputs: offset
@@ -636,7 +666,7 @@ struct WarpCore {
     template <bool CG = false>
     static __device__ __forceinline__ void decode_tile(const DecodeParams& p, const Extent& x, u64 t, const Fetch& f,
                                                        const u64* ex_tiles, const uint4* dict, const uint8_t* lens,
-                                                       WarpArea<K>& area, u32& err, u32* pk = nullptr) {
+                                                       Area& area, u32& err, u32* pk = nullptr) {
         const u32 lane = threadIdx.x & 31u;
         const u64 tile_start = (x.first_tile + t) * (u64)TILE;
         const u64 q0 = tile_start + (u64)lane * K;
@@ -644,6 +674,15 @@ struct WarpCore {
         // low word of the next tile's offset (lane 0 checks), in flight during the tile
         const bool chk = lane == 0u && t + 1 < x.n_tiles;
         const u32 ex_next = chk ? ld<CG>(reinterpret_cast<const u32*>(ex_tiles + t + 1)) : 0u;
+        // the tile's boundaries, clamped to the column's; the positions of
+        // the first of them are in flight while the tile is assembled
+        const u32 nb_col = p.n_strings + 1u;
+        const u32 b_hi = min(f.hi, nb_col);
+        u32 b_i = min(f.lo, nb_col) + lane;
+        u32 b_left = b_i < b_hi ? b_hi - b_i : 0u;
+        u32 pos[PB];
+#pragma unroll
+        for (int j = 0; j < PB; ++j) pos[j] = 32u * j < b_left ? ld_here(p.code_offsets + b_i + 32u * j) : 0u;
         R r;
         finish_load(p, x, q0, f.wv, f.fast, lens, r, pk);
         r.t = (u32)t;
@@ -731,74 +770,79 @@ struct WarpCore {
         const bool skip = p.size_only || tile_incl > p.capacity;
 
         // per-slot bytes and the offsets of every fourth slot, for the string offsets
+        u32 half = 0;   // bytes of the lane's first K/2 slots
         {
             u32 o = thr;
 #pragma unroll
             for (int j = 0; j < K / 4; ++j) {
+                if (j == K / 8) half = o - thr;
                 area.contrib[j][lane] = cw[j];
                 area.pre[j][lane] = o;
                 o += byte_sum(cw[j]);
             }
         }
-        Assembler as;
-        as.begin(p.out, tile_excl + thr, &area.fa[lane]);
-        if (!skip) {
-            if (!FSST) {
-                if (allv) assemble_onpair<true>(p, dict, r, as);
-                else assemble_onpair<false>(p, dict, r, as);
-            } else {
-                if (allv) assemble_fsst<true>(p, dict, r, cw, lit, as);
-                else assemble_fsst<false>(p, dict, r, cw, lit, as);
+        // Assembly in the warp's staging area, then whole-chunk stores.  A tile
+        // of more than CAP bytes takes rounds over consecutive lanes (a lane
+        // has at most 256 bytes).
+        u32* const stage = reinterpret_cast<u32*>(area.stage);
+        u32 rb = 0;
+        while (!skip && rb < tot) {
+            u32 end = tot;
+            if (tot - rb > (u32)(CAP - 16)) end = __reduce_max_sync(0xffffffffu, inc <= rb + (u32)(CAP - 16) ? inc : rb);
+            const bool in = thr >= rb && inc <= end;
+            const u64 G = tile_excl + rb;
+            const u32 off0 = (u32)(G & 15u), nb = off0 + (end - rb);
+            stage_free(lane);
+            StageWriter w0, w1;
+            w0.begin(stage, in ? off0 + (thr - rb) : 0u);
+            w1.begin(stage, in ? off0 + (thr + half - rb) : 0u);
+            if (in) {
+                if (allv) assemble<true>(p, dict, r, cw, lit, w0, w1);
+                else assemble<false>(p, dict, r, cw, lit, w0, w1);
             }
+            // the round's last word is completed by no lane: its bytes are only added
+            if (lane == 0u && (nb & 3u)) stage[nb >> 2] = 0u;
+            __syncwarp();
+            if (in) {
+                w0.finish();
+                w1.finish();
+            }
+            async_fence();
+            __syncwarp();
+            flush(area.stage, reinterpret_cast<uint4*>(p.out) + (G >> 4), off0, nb, lane);
+            rb = end;
         }
-        as.finish(produced > 0u && !skip);
-        area.meta[lane] = as.meta;
         __syncwarp();
 
-        // chunks shared between lanes; the tile's edge chunks, shared with
-        // the neighbouring tiles, are written bytewise by the whole warp
-        const bool wrote = !skip && produced > 0u;
-        Partial pd;
-        pd.pending = false;
-        if (wrote && (as.meta & FB_VALID))
-            combine_lanes(as.g, as.fb, 0u, (as.meta >> FB_HI_SHIFT) & 31u, (int)lane + 1, area.fa, area.meta, pd);
-        store_partials(pd);
-        pd.pending = false;
-        if (wrote && (as.meta & FA_VALID) && thr == 0u)
-            combine_lanes(as.dst0, area.fa[lane], (as.meta >> FA_LO_SHIFT) & 31u, (as.meta >> FA_HI_SHIFT) & 31u,
-                          (int)lane + 1, area.fa, area.meta, pd);
-        store_partials(pd);
-
-        // offsets of the strings whose boundaries the tile owns (the first
-        // PB*32 positions were fetched with the tile)
-        for (u32 i = f.lo + lane, j = 0; i < f.hi; i += 32, ++j) {
-            u64 pos;
-            if (j < (u32)PB) {
-                u32 v = f.pos[0];
+        // offsets of the strings whose boundaries the tile owns
+        while (b_left) {
 #pragma unroll
-                for (int m = 1; m < PB; ++m)
-                    if (j == (u32)m) v = f.pos[m];
-                pos = v;
-            } else {
-                pos = __ldg(p.code_offsets + i);
+            for (int j = 0; j < PB; ++j) {
+                if (32u * j >= b_left) break;
+                const u32 i = b_i + 32u * j;
+                u32 rel = 0;
+                u32 st = 0;
+                const u64 at = (u64)pos[j] - tile_start;   // wraps for positions before the tile
+                if (at < (u64)TILE) {
+                    const u32 sidx = (u32)at, sl = sidx / K, k = sidx % K;
+                    // offset of slot k's group of four, then the group's slots before k
+                    rel = area.pre[k >> 2][sl] + byte_sum(area.contrib[k >> 2][sl] & ((1u << (8u * (k & 3u))) - 1u));
+                    if (FSST) st = (area.lit_mask[sl] >> k) & 1u;
+                } else if (at == (u64)TILE) {
+                    rel = tot;
+                    st = tile_out_state;
+                    if (!last_tile) err |= ERRB_CORRUPT;
+                } else {
+                    err |= ERRB_CORRUPT;
+                }
+                if (st) err |= ERRB_CORRUPT;   // a string would start on a literal
+                if (!p.size_only) __stcs(p.out_offsets + i, (u32)tile_excl + rel);
             }
-            u64 rel = 0;
-            u32 st = 0;
-            if (pos < tile_start || pos > tile_start + TILE) {
-                err |= ERRB_CORRUPT;
-            } else if (pos == tile_start + TILE) {
-                rel = tile_incl - tile_excl;
-                st = tile_out_state;
-                if (!last_tile) err |= ERRB_CORRUPT;
-            } else {
-                const u32 sidx = (u32)(pos - tile_start);
-                const u32 j = sidx / K, k = sidx % K;
-                // offset of slot k's group of four, then the group's slots before k
-                rel = area.pre[k >> 2][j] + byte_sum(area.contrib[k >> 2][j] & ((1u << (8u * (k & 3u))) - 1u));
-                if (FSST) st = (area.lit_mask[j] >> k) & 1u;
-            }
-            if (st) err |= ERRB_CORRUPT;   // a string would start on a literal
-            if (!p.size_only) __stcs(p.out_offsets + i, (u32)(tile_excl + rel));
+            if (b_left <= 32u * PB) break;
+            b_i += 32u * PB;
+            b_left -= 32u * PB;
+#pragma unroll
+            for (int j = 0; j < PB; ++j) pos[j] = 32u * j < b_left ? ld_here(p.code_offsets + b_i + 32u * j) : 0u;
         }
         if (chk && ex_next != (u32)tile_incl) err |= ERRB_MISMATCH;
         __syncwarp();   // the area is reused by the next tile
@@ -806,28 +850,21 @@ struct WarpCore {
 
     // Decode the tiles t0, t0 + step, ... of the column (every lane of the
     // warp).  Software pipeline: while tile t decodes, the inputs of
-    // t + step are in flight and the boundaries of t + 2 step are being read.
+    // t + step are in flight.
     template <bool CG = false>
     static __device__ __forceinline__ void decode_tiles(const DecodeParams& p, const Extent& x, const u64* ex, u64 t,
                                                         u64 step, const uint4* dict, const uint8_t* lens,
-                                                        WarpArea<K>& area, u32& err, u32* pk) {
+                                                        Area& area, u32& err, u32* pk) {
         if (t >= x.n_tiles) return;
         Fetch cur;
-        u32 lo, hi, lo1 = 0, hi1 = 0;
-        bounds<CG>(p, t, lo, hi);
-        fetch<CG>(p, x, ex, t, lo, hi, cur);
-        if (t + step < x.n_tiles) bounds<CG>(p, t + step, lo1, hi1);
+        fetch<CG>(p, x, ex, t, cur);
         for (; t < x.n_tiles; t += step) {
             Fetch nxt;
-            const u64 tn = t + step, t2 = t + 2 * step;
-            u32 lo2 = 0, hi2 = 0;
-            if (tn < x.n_tiles) fetch<CG>(p, x, ex, tn, lo1, hi1, nxt);
-            if (t2 < x.n_tiles) bounds<CG>(p, t2, lo2, hi2);
+            if (t + step < x.n_tiles) fetch<CG>(p, x, ex, t + step, nxt);
             decode_tile<CG>(p, x, t, cur, ex, dict, lens, area, err, pk);
             cur = nxt;
-            lo1 = lo2;
-            hi1 = hi2;
         }
+        stage_free(threadIdx.x & 31u);   // shared memory outlives the copies from it
     }
 };
 
@@ -1097,26 +1134,26 @@ __global__ void __launch_bounds__(256) tiles_scan_kernel(const DecodeParams p, c
 // Pass 3: every warp decodes warp tiles on its own (grid-stride order).
 // ---------------------------------------------------------------------------
 template <int CODEC, int K, bool DSMEM, int NW, int MINB, int W = WarpCore<CODEC, K, DSMEM>::TOK8 ? 8 : 16,
-          bool PACKED = false>
+          bool PACKED = false, bool LSMEM = DSMEM>
 __global__ void __launch_bounds__(NW * 32, MINB) warp_decode_kernel(const DecodeParams p, const Extent* xp,
                                                                      const u64* ex) {
-    typedef WarpCore<CODEC, K, DSMEM, W, PACKED> C;
+    typedef WarpCore<CODEC, K, DSMEM, W, PACKED, LSMEM> C;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint4* s_dict = reinterpret_cast<uint4*>(smem_raw);
     uint8_t* s_lens = smem_raw + C::DICT_BYTES;
-    WarpArea<K>* areas = reinterpret_cast<WarpArea<K>*>(smem_raw + C::DICT_BYTES + (DSMEM ? C::LENS_BYTES : 0));
+    typename C::Area* areas = reinterpret_cast<typename C::Area*>(smem_raw + C::STAGED_BYTES);
     // packed codes: a scratch of PK_STRIDE words per lane after the warp areas
     u32* pk = PACKED ? reinterpret_cast<u32*>(areas + NW) + threadIdx.x * C::PK_STRIDE : nullptr;
     __shared__ __align__(8) u64 s_bar;
     if (C::BULK_STAGE) {
         C::stage_dict_bulk(p, s_dict, s_lens, &s_bar, NW * 32);
-    } else if (DSMEM) {
+    } else if (LSMEM) {
         C::stage_dict(p, s_dict, s_lens, NW * 32);
         __syncthreads();
     }
     grid_wait();   // the tile scan's offsets (the dictionary staging above overlapped it)
     const Extent x = *xp;
-    const uint8_t* lens = DSMEM ? s_lens : p.dict.lens;
+    const uint8_t* lens = LSMEM ? s_lens : p.dict.lens;
     u32 err = 0;
     C::decode_tiles(p, x, ex, (u64)blockIdx.x * NW + (threadIdx.x >> 5), (u64)gridDim.x * NW, s_dict, lens,
                     areas[threadIdx.x >> 5], err, pk);
@@ -1185,7 +1222,7 @@ __global__ void __launch_bounds__(NW * 32, 1) fused_decode_kernel(const DecodePa
     __shared__ Elem s_w[NW];
     uint4* s_dict = reinterpret_cast<uint4*>(smem_raw);
     uint8_t* s_lens = smem_raw + C::DICT_BYTES;
-    WarpArea<K>* areas = reinterpret_cast<WarpArea<K>*>(smem_raw + C::DICT_BYTES + (DSMEM ? C::LENS_BYTES : 0));
+    typename C::Area* areas = reinterpret_cast<typename C::Area*>(smem_raw + C::STAGED_BYTES);
     if (DSMEM) {
         C::stage_dict(p, s_dict, s_lens, NW * 32);
         __syncthreads();
