@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256) wbatch_scan_kernel(const BatchParams bp) 
 
 template <int CODEC, int K>
 __device__ __forceinline__ void decode_queue(const BatchParams& bp, int q, u64 t, u64 t_end, u64 W,
-                                             unsigned char* area_raw, SlotSrc& rs) {
+                                             unsigned char* area_raw, SlotSrc& rs, u64* bar, u32& phase) {
     typedef WarpCore<CODEC, K, false> C;
     const BatchQueue& Q = bp.q[q];
     typename C::Area& area = *reinterpret_cast<typename C::Area*>(area_raw);
@@ -178,14 +178,14 @@ __device__ __forceinline__ void decode_queue(const BatchParams& bp, int q, u64 t
     // software pipeline as in the single-column decode: while tile t decodes,
     // the inputs of t + W are in flight and the chunk of t + 2W is being read
     const SlotSrc* rc = Q.src + __ldg(Q.tile_chunk + t);
+    typename C::CodeBar cb{bar, phase};
     typename C::Fetch cur;
-    C::fetch(rc->p, rc->x, bp.ex + rc->wt_base, t - rc->tile_base, cur);
+    C::fetch(rc->p, rc->x, bp.ex + rc->wt_base, t - rc->tile_base, area, cb, cur);
     const SlotSrc* rn = t + W < t_end ? Q.src + __ldg(Q.tile_chunk + t + W) : nullptr;
     const SlotSrc* held = nullptr;   // the record copied into rs
     for (; t < t_end; t += W) {
         typename C::Fetch nxt;
         const u64 tn = t + W, t2 = t + 2 * W;
-        if (tn < t_end) C::fetch(rn->p, rn->x, bp.ex + rn->wt_base, tn - rn->tile_base, nxt);
         const SlotSrc* r2 = t2 < t_end ? Q.src + __ldg(Q.tile_chunk + t2) : nullptr;
         if (rc != held) {
             // the chunk's record into the warp's slot (the previous tile is done with it)
@@ -198,13 +198,22 @@ __device__ __forceinline__ void decode_queue(const BatchParams& bp, int q, u64 t
         // the error word's address is read before the tile: once the tile's
         // last __syncwarp() has passed, other lanes may overwrite the record
         unsigned* const err_word = rs.p.err_word;
-        C::decode_tile(rs.p, rs.x, t - rs.tile_base, cur, bp.ex + rs.wt_base, nullptr, rs.p.dict.lens, area, err);
+        C::decode_tile(rs.p, rs.x, t - rs.tile_base, cur, bp.ex + rs.wt_base, nullptr, rs.p.dict.lens, area, cb, err,
+                       [&] {
+                           if (tn < t_end)
+                               C::fetch(rn->p, rn->x, bp.ex + rn->wt_base, tn - rn->tile_base, area, cb, nxt);
+                       });
         if (err) atomicOr(err_word, err);
         cur = nxt;
         rc = rn;
         rn = r2;
     }
-    C::stage_free(lane);   // the area and the record slot are reused by the next queue
+    phase = cb.phase;
+    // the area and the record slot are reused by the next queue, whose bulk
+    // copies may land where this one stored
+    C::stage_free(lane);
+    async_fence();
+    __syncwarp();
 }
 
 // Bytes of a warp's scratch area (one layout serves every codec's queue).
@@ -229,10 +238,20 @@ __global__ void __launch_bounds__(NW * 32, MINB) wbatch_decode_kernel(const Batc
     // grid (contiguous ranges per block were tried: 14 % slower, the blocks'
     // ranges end unevenly).
     const u64 gw = (u64)blockIdx.x * NW + warp, W = (u64)gridDim.x * NW;
-    decode_queue<FP_ONPAIR16, K16>(bp, 0, gw, bp.q[0].n_tiles, W, mine, rs);
-    decode_queue<FP_ONPAIR12, K12>(bp, 1, gw, bp.q[1].n_tiles, W, mine, rs);
-    decode_queue<FP_FSST8, K8>(bp, 2, gw, bp.q[2].n_tiles, W, mine, rs);
-    decode_queue<FP_FSST12, K12>(bp, 3, gw, bp.q[3].n_tiles, W, mine, rs);
+    // one barrier per warp for the code copies of every queue, outside the
+    // areas (their layout changes with the codec)
+    __shared__ __align__(8) u64 s_code_bar[NW];
+    u64* bar = s_code_bar + warp;
+    if ((threadIdx.x & 31u) == 0u) {
+        mbar_init(bar, 1u);
+        mbar_init_fence();
+    }
+    __syncwarp();
+    u32 phase = 0u;
+    decode_queue<FP_ONPAIR16, K16>(bp, 0, gw, bp.q[0].n_tiles, W, mine, rs, bar, phase);
+    decode_queue<FP_ONPAIR12, K12>(bp, 1, gw, bp.q[1].n_tiles, W, mine, rs, bar, phase);
+    decode_queue<FP_FSST8, K8>(bp, 2, gw, bp.q[2].n_tiles, W, mine, rs, bar, phase);
+    decode_queue<FP_FSST12, K12>(bp, 3, gw, bp.q[3].n_tiles, W, mine, rs, bar, phase);
 }
 
 template <int K16, int K12, int K8, int NW>

@@ -173,28 +173,27 @@ cudaError_t launch_decode(int codec, const Variant& var, const DecodeParams& p_i
                                            stream);
     }
 
-    // warp tiles: index pass + reduce in one launch, tile scan, decode.  The
-    // first launch waits for everything before it (the previous call's decode
-    // still reads this workspace); the next two may start early and wait in
-    // the kernel for their predecessor.
-    const uint64_t n_wt_max = L.n_tiles;   // upper bound; the kernels read the true count from *xp
+    // warp tiles: index pass + reduce in one launch, tile scan, decode.  Each
+    // may start while the launch before it finishes and waits in the kernel
+    // before it reads that launch's results.
+    const uint64_t n_wt_max = L.n_tiles;   // upper bound; the kernels compute the true count
     uint64_t rg = (n_wt_max + 7) / 8;
     const uint64_t rg_cap = (uint64_t)sms * 8;
     if (rg > rg_cap) rg = rg_cap;
-    const Extent* cxp = xp;
     u32 ib32 = (u32)ib;
     void* rargs[] = {(void*)&p, (void*)&xp, (void*)&agg, (void*)&ib32};
-    e = cudaLaunchKernel(var.reduce, dim3((unsigned)(rg + ib)), dim3(256), rargs, 0, stream);
+    e = launch_after(var.reduce, dim3((unsigned)(rg + ib)), dim3(256), rargs, 0, stream);
     if (e != cudaSuccess) return e;
     uint64_t sg = n_wt_max / kScanTile + 1;
     if (sg > (uint64_t)sms * 2) sg = (uint64_t)sms * 2;
     const u64* cagg = agg;
     unsigned long long* st = p.tile_status;
-    void* sargs[] = {(void*)&p, (void*)&cxp, (void*)&cagg, (void*)&ex, (void*)&st};
+    u32 tile32 = (u32)tile;
+    void* sargs[] = {(void*)&p, (void*)&tile32, (void*)&cagg, (void*)&ex, (void*)&st};
     e = launch_after(var.scan, dim3((unsigned)sg), dim3(256), sargs, 0, stream);
     if (e != cudaSuccess) return e;
     const u64* cex = ex;
-    void* dargs[] = {(void*)&p, (void*)&cxp, (void*)&cex};
+    void* dargs[] = {(void*)&p, (void*)&cex};
     const int nw = var.threads / 32;
     uint64_t dg = (n_wt_max + nw - 1) / nw;
     if (dg > (uint64_t)grid) dg = (uint64_t)grid;

@@ -81,6 +81,33 @@ __device__ __forceinline__ void bar_arrive(u32 id, u32 n) {
 // are visible (at once for a kernel launched without the attribute), and
 // grid_release() lets the next kernel start launching.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// What a launch before this one may have written while this one was already
+// running (results of our own passes; the caller's column, in the first
+// launch of a call) is read after grid_wait() through after_wait() pointers
+// or in_order() loads, never with __ldg(): the read-only path may be read
+// ahead of the wait.
+template <class T>
+__device__ __forceinline__ const T* after_wait(const T* a) {
+    const T* r;
+    asm volatile("mov.b64 %0, %1;" : "=l"(r) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ u32 in_order(const u32* a) {
+    u32 v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(a));
+    return v;
+}
+// The same past L1 (words that other SMs wrote in this launch or the one before).
+__device__ __forceinline__ u32 in_order_l2(const u32* a) {
+    u32 v;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(a));
+    return v;
+}
+__device__ __forceinline__ u64 in_order_l2(const u64* a) {
+    u64 v;
+    asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(v) : "l"(a));
+    return v;
+}
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ u64 status_word(u64 flag, u32 epoch, u64 payload) {
@@ -478,8 +505,8 @@ __device__ void combine_and_store(uint4* chunk, uint4 acc, u32 lo, u32 hi, int m
 // The column's slot range [c_begin, c_end) from code_offsets[0] and
 // code_offsets[n], clamped to the code buffer (x.bad when it had to be).
 __device__ __forceinline__ void slot_range(const DecodeParams& p, Extent& x) {
-    x.c_begin = __ldg(p.code_offsets);
-    x.c_end = __ldg(p.code_offsets + p.n_strings);
+    x.c_begin = in_order(p.code_offsets);
+    x.c_end = in_order(p.code_offsets + p.n_strings);
     x.bad = 0u;
     if (x.c_end > p.max_slots) { x.c_end = p.max_slots; x.bad = 1u; }
     if (x.c_begin > x.c_end) { x.c_begin = x.c_end; x.bad = 1u; }
@@ -538,7 +565,7 @@ __device__ __forceinline__ void index_groups(const DecodeParams& p, const Extent
 #pragma unroll
         for (int k = 0; k <= kIdxGroup; ++k) {
             const u64 i = i0 + k - 1;   // v[0] is boundary i0 - 1
-            v[k] = (k > 0 || i0 > 0) && i < i_end ? __ldg(p.code_offsets + i) : 0u;
+            v[k] = (k > 0 || i0 > 0) && i < i_end ? in_order(p.code_offsets + i) : 0u;
         }
 #pragma unroll
         for (int k = 0; k < kIdxGroup; ++k)

@@ -97,7 +97,7 @@ struct Path {
         return (size_t)C::STAGED_BYTES + kSidecarWarps * sizeof(typename C::Area);
     }
     static const void* decode_kernel() {
-        return (const void*)&warp_decode_kernel<CODEC, K, DSMEM, kSidecarWarps, 1, W, false, true>;
+        return (const void*)&warp_decode_kernel<CODEC, K, DSMEM, kSidecarWarps, 1, W, false, true, false>;
     }
     // Index pass in blocks [0, ib), reduce in the next rg blocks (rg = 0: index only).
     static cudaError_t index_reduce(const DecodeParams& p, Extent* xp, u64* agg, uint64_t ib, uint64_t rg,
@@ -107,15 +107,15 @@ struct Path {
         return cudaLaunchKernel((const void*)&reduce_kernel<CODEC, K, DSMEM>, dim3((unsigned)(ib + rg)), dim3(256),
                                 args, 0, s);
     }
-    static cudaError_t scan(const DecodeParams& p, const Extent* xp, const u64* agg, u64* ex, uint64_t grid,
-                            cudaStream_t s) {
+    static cudaError_t scan(const DecodeParams& p, const u64* agg, u64* ex, uint64_t grid, cudaStream_t s) {
         unsigned long long* st = p.tile_status;
-        void* args[] = {(void*)&p, (void*)&xp, (void*)&agg, (void*)&ex, (void*)&st};
+        u32 tile = C::TILE;
+        void* args[] = {(void*)&p, (void*)&tile, (void*)&agg, (void*)&ex, (void*)&st};
         return cudaLaunchKernel((const void*)&tiles_scan_kernel<CODEC == FP_FSST8>, dim3((unsigned)grid), dim3(256),
                                 args, 0, s);
     }
-    static cudaError_t decode(const DecodeParams& p, const Extent* xp, const u64* ex, uint64_t grid, cudaStream_t s) {
-        void* args[] = {(void*)&p, (void*)&xp, (void*)&ex};
+    static cudaError_t decode(const DecodeParams& p, const u64* ex, uint64_t grid, cudaStream_t s) {
+        void* args[] = {(void*)&p, (void*)&ex};
         return cudaLaunchKernel(decode_kernel(), dim3((unsigned)grid), dim3(kSidecarWarps * 32), args, decode_smem(),
                                 s);
     }
@@ -209,7 +209,7 @@ cudaError_t build_launches(const DecodeParams& p, char* scratch, const Layout& L
     if (e != cudaSuccess) return e;
     uint64_t sg = L.n_tiles / kScanTile + 1;
     if (sg > (uint64_t)sms * 2) sg = (uint64_t)sms * 2;
-    return P::scan(p, xp, agg, ex, sg, s);
+    return P::scan(p, agg, ex, sg, s);
 }
 
 template <int CODEC>
@@ -224,7 +224,7 @@ cudaError_t decode_launches(const DecodeParams& p, char* scratch, const Layout& 
     if (e != cudaSuccess) return e;
     uint64_t grid = (L.n_tiles + kSidecarWarps - 1) / kSidecarWarps;
     if (grid > (uint64_t)sms) grid = (uint64_t)sms;
-    return P::decode(p, xp, sidecar + 1, grid, s);
+    return P::decode(p, sidecar + 1, grid, s);
 }
 
 }  // namespace

@@ -69,8 +69,7 @@ Variant make_packed_variant() {
     v.threads = NW * 32;
     v.slots_per_thread = K;
     v.dict_smem = DSMEM ? 1 : 0;
-    v.smem_bytes = (size_t)C::STAGED_BYTES + NW * sizeof(typename C::Area) +
-                   (size_t)NW * 32 * C::PK_STRIDE * sizeof(u32);
+    v.smem_bytes = (size_t)C::STAGED_BYTES + NW * sizeof(typename C::Area);
     v.kernel = (const void*)&warp_decode_kernel<CODEC, K, DSMEM, NW, 1, W, true, true>;
     v.warp_tiles = 1;
     v.reduce = (const void*)&reduce_kernel<CODEC, K, DSMEM, true>;

@@ -116,9 +116,11 @@ struct StageWriter {
 // decoded bytes, at the alignment they have in the output, so that the whole
 // 16-byte chunks leave by one bulk copy per tile (no store instructions, and
 // no scattered lines in L1).
-template <int K, int CAP>
+template <int K, int CAP, int CODE_BYTES, int SCRATCH>
 struct WarpArea {
     uint4 stage[CAP / 16 + 1];
+    // code bytes of the tile to decode next (bulk copy), or the unpack's scratch (packed codes)
+    uint4 codes[CODE_BYTES + SCRATCH ? (CODE_BYTES + SCRATCH) / 16 : 1];
     u32 pre[K / 4][32];     // tile-relative output offset of slot 4m of each lane
     u32 contrib[K / 4][32]; // bytes each slot produced, one byte per slot
     u32 lit_mask[32];       // FSST-8: bit k = slot k holds a literal byte
@@ -161,7 +163,15 @@ struct WarpCore {
     // tokens of 7.5 bytes: 3.8 KB; 1,024 FSST symbols: 4.6 KB); less where
     // the dictionary is read through L1, which shares the SM's memory.
     static constexpr int CAP = DSMEM ? 6144 : 4096;
-    typedef WarpArea<K, CAP> Area;
+    static constexpr int TILE_BYTES = TILE * WBITS / 8;   // code bytes of a tile
+    // The next tile's codes come by a bulk copy into the warp's area (32-slot
+    // lanes), or into registers.  The copy frees 8 to 12 registers and
+    // writes each line once where lanes 32 or 48 bytes apart touch it several
+    // times; 32-slot lanes are short of registers (FSST-8 16M strings 601 ->
+    // 576 us per call, FSST-12 documents 114 -> 105), 16-slot lanes are not
+    // and only pay the wait (OnPair-12 10M 648 -> 659).
+    static constexpr bool BULK_CODES = K == 32;
+    typedef WarpArea<K, CAP, BULK_CODES ? TILE_BYTES : 0, PACKED ? 32 * PK_STRIDE * 4 : 0> Area;
     static constexpr int LENS_BYTES = LSMEM ? kTable : 0;
     static constexpr int STAGED_BYTES = DICT_BYTES + LENS_BYTES;   // tables in front of the warp areas
     typedef TileRegs<CODEC, K> R;
@@ -221,6 +231,15 @@ struct WarpCore {
             }
         }
         return true;
+    }
+
+    // The same words from the tile's bulk-copied code bytes.
+    static __device__ __forceinline__ void load_staged(const uint4* codes, u32 lane, u32 (&wv)[LANE_WORDS]) {
+#pragma unroll
+        for (int v = 0; v < LANE_BYTES / 16; ++v) {
+            const uint4 a = codes[lane * (LANE_BYTES / 16) + v];
+            wv[4 * v] = a.x; wv[4 * v + 1] = a.y; wv[4 * v + 2] = a.z; wv[4 * v + 3] = a.w;
+        }
     }
 
     static __device__ void load_guarded(const DecodeParams& p, u64 q0, R& r) {
@@ -308,18 +327,20 @@ struct WarpCore {
         }
     }
 
-    // Codes (from words load_fast() fetched, or guarded loads), the slots
-    // inside the column and their token lengths.  `pk`: the lane's scratch
-    // (packed codes only).
-    static __device__ __forceinline__ void finish_load(const DecodeParams& p, const Extent& x, u64 q0,
-                                                       const u32 (&wv)[LANE_WORDS], bool fast, const uint8_t* lens,
-                                                       R& r, u32* pk = nullptr) {
+    // Codes, from words load_fast() or load_staged() fetched or by guarded
+    // loads.  `pk`: the lane's scratch (packed codes only).
+    static __device__ __forceinline__ void unpack(const DecodeParams& p, u64 q0, const u32 (&wv)[LANE_WORDS], bool fast,
+                                                  R& r, u32* pk = nullptr) {
         if (fast) {
             if (PACKED) unpack_packed(wv, (u32)((q0 * p.packed_bits) & 31u), p.packed_bits, pk, r);
             else unpack_words(wv, r);
         } else {
             load_guarded(p, q0, r);
         }
+    }
+
+    // The slots of the lane inside the column.
+    static __device__ __forceinline__ void mark_valid(const Extent& x, u64 q0, R& r) {
         if (q0 >= x.c_begin && q0 + K <= x.c_end) {
             r.valid = full_mask();
         } else {
@@ -331,6 +352,14 @@ struct WarpCore {
             }
             r.valid = v;
         }
+    }
+
+    // The codes, the slots inside the column and their token lengths.
+    static __device__ __forceinline__ void finish_load(const DecodeParams& p, const Extent& x, u64 q0,
+                                                       const u32 (&wv)[LANE_WORDS], bool fast, const uint8_t* lens,
+                                                       R& r, u32* pk = nullptr) {
+        unpack(p, q0, wv, fast, r, pk);
+        mark_valid(x, q0, r);
 #pragma unroll
         for (int j = 0; j < K / 4; ++j) {
             u32 w = 0;
@@ -629,64 +658,89 @@ struct WarpCore {
         return (x.first_tile + t) * (u64)TILE + (u64)(threadIdx.x & 31u) * K;
     }
 
-    // Inputs of a warp tile fetched ahead of its decode: the lane's code
-    // words, the tile's scanned offset, its string boundaries [lo, hi) (as
-    // stored: clamped where they are used, so that nothing waits for the
-    // loads here).
+    // Inputs of a warp tile fetched ahead of its decode: its codes (`in` is
+    // false for a lane whose codes run past the code buffer: guarded loads
+    // instead; with BULK_CODES for a whole tile), the tile's scanned offset
+    // and its string boundaries [lo, hi) (as stored: clamped where they are
+    // used, so that nothing waits for the loads here).
     struct Fetch {
-        u32 wv[LANE_WORDS];
-        bool fast;
+        u32 wv[BULK_CODES ? 1 : LANE_WORDS];
+        bool in;
         u64 ex;
         u32 lo, hi;
+    };
+    // The warp's mbarrier for those copies and the phase of the next one.
+    struct CodeBar {
+        u64* bar;
+        u32 phase;
+        // Every lane of the warp calls it, before the first fetch().
+        __device__ __forceinline__ void init(u64* b) {
+            bar = b;
+            phase = 0u;
+            if ((threadIdx.x & 31u) == 0u) {
+                mbar_init(bar, 1u);
+                mbar_init_fence();
+            }
+            __syncwarp();
+        }
     };
     // Rounds of 32 boundaries whose code_offsets are in flight together.
     static constexpr int PB = K / 8;
 
-    // Loads of data written by this launch's earlier phases (the one-launch
-    // decode, CG) bypass L1; otherwise the read-only path.
-    template <bool CG, class T>
-    static __device__ __forceinline__ T ld(const T* a) { return CG ? __ldcg(a) : __ldg(a); }
-
-    // Issue the loads of tile t.
-    template <bool CG = false>
-    static __device__ __forceinline__ void fetch(const DecodeParams& p, const Extent& x, const u64* ex, u64 t, Fetch& f) {
-        f.fast = load_fast(p, lane_q0(x, t), f.wv);
-        f.ex = ld<CG>(ex + t);
-        f.lo = ld<CG>(p.first + t);
-        f.hi = ld<CG>(p.first + t + 1);
+    // Issue the loads of tile t (every lane of the warp, the tile before it
+    // read from area.codes): its codes, which are the caller's input, and
+    // what the passes before the decode made.
+    static __device__ __forceinline__ void fetch_codes(const DecodeParams& p, const Extent& x, u64 t, Area& area,
+                                                       const CodeBar& cb, Fetch& f) {
+        if constexpr (BULK_CODES) {
+            const u64 b0 = (x.first_tile + t) * TILE_BYTES;   // a multiple of 16, as TILE_BYTES is
+            f.in = b0 + TILE_BYTES <= p.codes_bytes;
+            if (f.in && (threadIdx.x & 31u) == 0u) {
+                mbar_expect_tx(cb.bar, (u32)TILE_BYTES);
+                bulk_g2s(area.codes, p.codes + b0, (u32)TILE_BYTES, cb.bar);
+                mbar_arrive(cb.bar);
+            }
+        } else {
+            f.in = load_fast(p, lane_q0(x, t), f.wv);
+        }
+    }
+    // The launches (or phases) before this one wrote these while it was
+    // already running.
+    static __device__ __forceinline__ void fetch_scanned(const u64* ex, const u32* first, u64 t, Fetch& f) {
+        f.ex = in_order_l2(ex + t);
+        f.lo = in_order_l2(first + t);
+        f.hi = in_order_l2(first + t + 1);
+    }
+    static __device__ __forceinline__ void fetch(const DecodeParams& p, const Extent& x, const u64* ex, u64 t,
+                                                 Area& area, const CodeBar& cb, Fetch& f) {
+        fetch_codes(p, x, t, area, cb, f);
+        fetch_scanned(ex, p.first, t, f);
     }
 
-    // Decode warp tile t of column (p, x) from its fetched inputs: offset
-    // and entering escape state (from the tile scan), code words, string
-    // boundaries.  `area` is the warp's scratch.  `ex_tiles` holds the
-    // column's scanned tile offsets (f.ex = ex_tiles[t]): the tile's own
-    // byte total, recomputed here, must bring it to ex_tiles[t + 1], else
-    // ERRB_MISMATCH is raised (a self-check of the two passes, one load
-    // per tile).
-    template <bool CG = false>
-    static __device__ __forceinline__ void decode_tile(const DecodeParams& p, const Extent& x, u64 t, const Fetch& f,
-                                                       const u64* ex_tiles, const uint4* dict, const uint8_t* lens,
-                                                       Area& area, u32& err, u32* pk = nullptr) {
+    // The first boundaries of a tile: positions in flight while it is
+    // assembled.
+    struct Strings {
+        u32 first, left;   // the lane's first boundary, boundaries from it to the tile's end
+        u32 pos[PB];
+    };
+    // Boundaries [lo, hi), clamped to the column's; issues the loads.
+    static __device__ __forceinline__ void strings_begin(const DecodeParams& p, u32 lo, u32 hi, Strings& sb) {
+        const u32 nb_col = p.n_strings + 1u;
+        hi = min(hi, nb_col);
+        sb.first = min(lo, nb_col) + (threadIdx.x & 31u);
+        sb.left = sb.first < hi ? hi - sb.first : 0u;
+#pragma unroll
+        for (int j = 0; j < PB; ++j) sb.pos[j] = 32u * j < sb.left ? ld_here(p.code_offsets + sb.first + 32u * j) : 0u;
+    }
+
+    // Assemble warp tile t of column (p, x) from its codes and token lengths
+    // (r): the bytes, then the offsets of the strings whose boundaries it
+    // owns.  `ex` is its output offset and entering escape state; returns
+    // the same for the tile after it.
+    static __device__ __forceinline__ u64 assemble_tile(const DecodeParams& p, const Extent& x, u64 t, R& r, u64 ex,
+                                                        Strings& sb, const uint4* dict, Area& area, u32& err) {
         const u32 lane = threadIdx.x & 31u;
         const u64 tile_start = (x.first_tile + t) * (u64)TILE;
-        const u64 q0 = tile_start + (u64)lane * K;
-        const u64 ex = f.ex;
-        // low word of the next tile's offset (lane 0 checks), in flight during the tile
-        const bool chk = lane == 0u && t + 1 < x.n_tiles;
-        const u32 ex_next = chk ? ld<CG>(reinterpret_cast<const u32*>(ex_tiles + t + 1)) : 0u;
-        // the tile's boundaries, clamped to the column's; the positions of
-        // the first of them are in flight while the tile is assembled
-        const u32 nb_col = p.n_strings + 1u;
-        const u32 b_hi = min(f.hi, nb_col);
-        u32 b_i = min(f.lo, nb_col) + lane;
-        u32 b_left = b_i < b_hi ? b_hi - b_i : 0u;
-        u32 pos[PB];
-#pragma unroll
-        for (int j = 0; j < PB; ++j) pos[j] = 32u * j < b_left ? ld_here(p.code_offsets + b_i + 32u * j) : 0u;
-        R r;
-        finish_load(p, x, q0, f.wv, f.fast, lens, r, pk);
-        r.t = (u32)t;
-        r.tile_start = tile_start;
         const bool allv = (r.valid == full_mask());
         const u64 tile_excl = ex & 0x7fffffffffffffffull;
         const u32 s_tile = FSST ? (u32)(ex >> 63) : 0u;
@@ -814,15 +868,16 @@ struct WarpCore {
         }
         __syncwarp();
 
+        u32 first = sb.first, left = sb.left;
         // offsets of the strings whose boundaries the tile owns
-        while (b_left) {
+        while (left) {
 #pragma unroll
             for (int j = 0; j < PB; ++j) {
-                if (32u * j >= b_left) break;
-                const u32 i = b_i + 32u * j;
+                if (32u * j >= left) break;
+                const u32 i = first + 32u * j;
                 u32 rel = 0;
                 u32 st = 0;
-                const u64 at = (u64)pos[j] - tile_start;   // wraps for positions before the tile
+                const u64 at = (u64)sb.pos[j] - tile_start;   // wraps for positions before the tile
                 if (at < (u64)TILE) {
                     const u32 sidx = (u32)at, sl = sidx / K, k = sidx % K;
                     // offset of slot k's group of four, then the group's slots before k
@@ -838,30 +893,80 @@ struct WarpCore {
                 if (st) err |= ERRB_CORRUPT;   // a string would start on a literal
                 if (!p.size_only) __stcs(p.out_offsets + i, (u32)tile_excl + rel);
             }
-            if (b_left <= 32u * PB) break;
-            b_i += 32u * PB;
-            b_left -= 32u * PB;
+            if (left <= 32u * PB) break;
+            first += 32u * PB;
+            left -= 32u * PB;
 #pragma unroll
-            for (int j = 0; j < PB; ++j) pos[j] = 32u * j < b_left ? ld_here(p.code_offsets + b_i + 32u * j) : 0u;
+            for (int j = 0; j < PB; ++j) sb.pos[j] = 32u * j < left ? ld_here(p.code_offsets + first + 32u * j) : 0u;
         }
-        if (chk && ex_next != (u32)tile_incl) err |= ERRB_MISMATCH;
-        __syncwarp();   // the area is reused by the next tile
+        __syncwarp();   // the areas are reused by the next tile
+        return tile_incl | ((u64)tile_out_state << 63);
+    }
+
+    // Decode warp tile t of column (p, x) from its fetched inputs: offset
+    // and entering escape state (from the tile scan), code words, string
+    // boundaries.  `area` is the warp's scratch.  `ex_tiles` holds the
+    // column's scanned tile offsets (f.ex = ex_tiles[t]): the tile's own
+    // byte total, recomputed here, must bring it to ex_tiles[t + 1], else
+    // ERRB_MISMATCH is raised (a self-check of the two passes, one load
+    // per tile).
+    // `next` issues the fetch of the warp's next tile (it is called once
+    // area.codes is free).
+    template <class Next>
+    static __device__ __forceinline__ void decode_tile(const DecodeParams& p, const Extent& x, u64 t, const Fetch& f,
+                                                       const u64* ex_tiles, const uint4* dict, const uint8_t* lens,
+                                                       Area& area, CodeBar& cb, u32& err, Next&& next) {
+        const u32 lane = threadIdx.x & 31u;
+        const u64 q0 = lane_q0(x, t);
+        const u64 ex = f.ex;
+        // low word of the next tile's offset (lane 0 checks), in flight during the tile
+        const bool chk = lane == 0u && t + 1 < x.n_tiles;
+        const u32 ex_next = chk ? in_order_l2(reinterpret_cast<const u32*>(ex_tiles + t + 1)) : 0u;
+        Strings sb;
+        strings_begin(p, f.lo, f.hi, sb);
+        R r;
+        if constexpr (BULK_CODES) {
+            u32 wv[LANE_WORDS];
+            const bool in = f.in;
+            if (in) {
+                mbar_wait(cb.bar, cb.phase, p.ws);
+                cb.phase ^= 1u;
+                load_staged(area.codes, lane, wv);
+            }
+            __syncwarp();   // the codes have left the area
+            next();
+            finish_load(p, x, q0, wv, in, lens, r);
+        } else {
+            next();
+            finish_load(p, x, q0, f.wv, f.in, lens, r, reinterpret_cast<u32*>(area.codes) + lane * PK_STRIDE);
+        }
+        const u64 next_ex = assemble_tile(p, x, t, r, ex, sb, dict, area, err);
+        if (chk && ex_next != (u32)next_ex) err |= ERRB_MISMATCH;
     }
 
     // Decode the tiles t0, t0 + step, ... of the column (every lane of the
     // warp).  Software pipeline: while tile t decodes, the inputs of
     // t + step are in flight.
-    template <bool CG = false>
     static __device__ __forceinline__ void decode_tiles(const DecodeParams& p, const Extent& x, const u64* ex, u64 t,
                                                         u64 step, const uint4* dict, const uint8_t* lens,
-                                                        Area& area, u32& err, u32* pk) {
-        if (t >= x.n_tiles) return;
+                                                        Area& area, u64* bar, u32& err) {
+        if (t >= x.n_tiles) {
+            grid_wait();
+            return;
+        }
+        CodeBar cb;
+        cb.init(bar);
         Fetch cur;
-        fetch<CG>(p, x, ex, t, cur);
+        fetch_codes(p, x, t, area, cb, cur);
+        grid_wait();   // the launch before (none before a cooperative launch's phases)
+        fetch_scanned(ex, p.first, t, cur);
         for (; t < x.n_tiles; t += step) {
             Fetch nxt;
-            if (t + step < x.n_tiles) fetch<CG>(p, x, ex, t + step, nxt);
-            decode_tile<CG>(p, x, t, cur, ex, dict, lens, area, err, pk);
+            decode_tile(p, x, t, cur, ex, dict, lens, area, cb, err, [&] {
+                if (t + step >= x.n_tiles) return;
+                fetch_codes(p, x, t + step, area, cb, nxt);
+                fetch_scanned(ex, p.first, t + step, nxt);
+            });
             cur = nxt;
         }
         stage_free(threadIdx.x & 31u);   // shared memory outlives the copies from it
@@ -886,11 +991,19 @@ struct ReduceShape {
 };
 
 template <int CODEC, int K, bool DSMEM, bool PACKED = false>
-__global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kernel(const DecodeParams p, Extent* xp,
+__global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kernel(const DecodeParams pp, Extent* xp,
                                                                                   u64* agg, u32 index_blocks) {
     typedef WarpCore<CODEC, K, DSMEM, WarpCore<CODEC, K, DSMEM>::TOK8 ? 8 : 16, PACKED> C;
     __shared__ __align__(16) uint8_t s_lens[DSMEM ? C::LENS_BYTES : 16];
     __shared__ __align__(16) u32 s_pk[PACKED ? 256 * C::PK_STRIDE : 2];   // packed codes: per-lane scratch
+    if (DSMEM && blockIdx.x >= index_blocks) {
+        // the dictionary is older than any launch this one may overlap
+        const uint4* src = reinterpret_cast<const uint4*>(pp.dict.lens);
+        for (int i = threadIdx.x; i < C::LENS_BYTES / 16; i += blockDim.x) reinterpret_cast<uint4*>(s_lens)[i] = __ldg(src + i);
+    }
+    grid_wait();      // the launch before: the column may be its output, the workspace its scratch
+    DecodeParams p = pp;
+    p.codes = after_wait(pp.codes);
     grid_release();   // the next launch may be scheduled as these blocks retire (it waits for their results)
     if (blockIdx.x < index_blocks) {
         const Extent x = column_extent(p, C::TILE);
@@ -900,11 +1013,7 @@ __global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kerne
                      const_cast<u32*>(p.first));
         return;
     }
-    if (DSMEM) {
-        const uint4* src = reinterpret_cast<const uint4*>(p.dict.lens);
-        for (int i = threadIdx.x; i < C::LENS_BYTES / 16; i += blockDim.x) reinterpret_cast<uint4*>(s_lens)[i] = __ldg(src + i);
-        __syncthreads();
-    }
+    if (DSMEM) __syncthreads();
     const Extent x = column_extent(p, C::TILE);
     const uint8_t* lens = DSMEM ? s_lens : p.dict.lens;
     const u32 lane = threadIdx.x & 31u;
@@ -1106,19 +1215,33 @@ __device__ __forceinline__ void scan_block(const DecodeParams& p, const u64* agg
     __syncthreads();   // shared words are rewritten for the next ticket
 }
 
+// The launch state the tile scan leaves behind (its tickets, the launch tag of
+// the look-back words, the stall settings), renewed by one thread of the
+// decode after it: the scan's blocks need not count themselves out.
+__device__ __forceinline__ void renew_launch(WsHeader* ws) {
+    ws->tile_counter = 0;
+    ws->abort = 0;
+    ws->spin_limit = 0;
+    ws->bar_count = 0;
+    const u32 ne = (ws->epoch + 1u) & kEpochMask;
+    ws->epoch = ne ? ne : 1u;
+}
+
+// Everything that does not depend on the reduce (the first ticket, the launch
+// tag, the column's extent) is fetched while the reduce still runs: on a
+// small column the scan is a chain of global round trips.
 template <bool FSST>
-__global__ void __launch_bounds__(256) tiles_scan_kernel(const DecodeParams p, const Extent* xp, const u64* agg,
-                                                         u64* ex, unsigned long long* status) {
+__global__ void __launch_bounds__(256) tiles_scan_kernel(const DecodeParams p, u32 tile, const u64* agg, u64* ex,
+                                                         unsigned long long* status) {
     __shared__ ScanShared sh;
     WsHeader* ws = p.ws;
     grid_release();   // the decode may start launching (its blocks stage the dictionary, then wait)
-    grid_wait();      // the reduce's elements and extent
-    const Extent x = *xp;
+    if (threadIdx.x == 0) sh.ticket = atomicAdd(&ws->tile_counter, 1u);
     const u32 epoch = *(volatile u32*)&ws->epoch;
-    const u64 n = x.n_tiles;
+    const u64 n = column_extent(p, tile).n_tiles;
     const u64 n_blocks = (n + kScanTile - 1) / kScanTile;
+    grid_wait();      // the reduce's elements
     for (;;) {
-        if (threadIdx.x == 0) sh.ticket = atomicAdd(&ws->tile_counter, 1u);
         __syncthreads();
         const u64 b = sh.ticket;
         if (b >= n_blocks) break;
@@ -1126,37 +1249,37 @@ __global__ void __launch_bounds__(256) tiles_scan_kernel(const DecodeParams p, c
         // with a block per scan block the first tickets cover them all: no
         // second ticket (one atomic round trip less at the end of the scan)
         if ((u64)gridDim.x >= n_blocks) break;
+        if (threadIdx.x == 0) sh.ticket = atomicAdd(&ws->tile_counter, 1u);
     }
-    finish_launch(ws, epoch);
 }
 
 // ---------------------------------------------------------------------------
 // Pass 3: every warp decodes warp tiles on its own (grid-stride order).
 // ---------------------------------------------------------------------------
 template <int CODEC, int K, bool DSMEM, int NW, int MINB, int W = WarpCore<CODEC, K, DSMEM>::TOK8 ? 8 : 16,
-          bool PACKED = false, bool LSMEM = DSMEM>
-__global__ void __launch_bounds__(NW * 32, MINB) warp_decode_kernel(const DecodeParams p, const Extent* xp,
-                                                                     const u64* ex) {
+          bool PACKED = false, bool LSMEM = DSMEM, bool RENEW = true>
+__global__ void __launch_bounds__(NW * 32, MINB) warp_decode_kernel(const DecodeParams p, const u64* ex) {
     typedef WarpCore<CODEC, K, DSMEM, W, PACKED, LSMEM> C;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint4* s_dict = reinterpret_cast<uint4*>(smem_raw);
     uint8_t* s_lens = smem_raw + C::DICT_BYTES;
     typename C::Area* areas = reinterpret_cast<typename C::Area*>(smem_raw + C::STAGED_BYTES);
-    // packed codes: a scratch of PK_STRIDE words per lane after the warp areas
-    u32* pk = PACKED ? reinterpret_cast<u32*>(areas + NW) + threadIdx.x * C::PK_STRIDE : nullptr;
     __shared__ __align__(8) u64 s_bar;
+    __shared__ __align__(8) u64 s_code_bar[NW];
     if (C::BULK_STAGE) {
         C::stage_dict_bulk(p, s_dict, s_lens, &s_bar, NW * 32);
     } else if (LSMEM) {
         C::stage_dict(p, s_dict, s_lens, NW * 32);
         __syncthreads();
     }
-    grid_wait();   // the tile scan's offsets (the dictionary staging above overlapped it)
-    const Extent x = *xp;
+    const Extent x = column_extent(p, C::TILE);
     const uint8_t* lens = LSMEM ? s_lens : p.dict.lens;
     u32 err = 0;
+    // decode_tiles() fetches the first tile's codes, then waits for the tile
+    // scan's offsets: staging and fetch overlap the scan
     C::decode_tiles(p, x, ex, (u64)blockIdx.x * NW + (threadIdx.x >> 5), (u64)gridDim.x * NW, s_dict, lens,
-                    areas[threadIdx.x >> 5], err, pk);
+                    areas[threadIdx.x >> 5], s_code_bar + (threadIdx.x >> 5), err);
+    if (RENEW && blockIdx.x == 0 && threadIdx.x == 0) renew_launch(p.ws);
     if (err) atomicOr(p.err_word, err);
 }
 
@@ -1220,6 +1343,7 @@ __global__ void __launch_bounds__(NW * 32, 1) fused_decode_kernel(const DecodePa
     typedef WarpCore<CODEC, K, DSMEM, W> C;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ Elem s_w[NW];
+    __shared__ __align__(8) u64 s_code_bar[NW];
     uint4* s_dict = reinterpret_cast<uint4*>(smem_raw);
     uint8_t* s_lens = smem_raw + C::DICT_BYTES;
     typename C::Area* areas = reinterpret_cast<typename C::Area*>(smem_raw + C::STAGED_BYTES);
@@ -1251,7 +1375,8 @@ __global__ void __launch_bounds__(NW * 32, 1) fused_decode_kernel(const DecodePa
     if (blockIdx.x == 0) block_scan_tiles<C::FSST, NW * 32>(p, agg, ex, x.n_tiles, s_w);
     grid_barrier(p.ws);
     // phase 3
-    C::template decode_tiles<true>(p, x, ex, gwarp, gwarps, s_dict, lens, areas[threadIdx.x >> 5], err, nullptr);
+    C::decode_tiles(p, x, ex, gwarp, gwarps, s_dict, lens, areas[threadIdx.x >> 5],
+                                   s_code_bar + (threadIdx.x >> 5), err);
     if (err) atomicOr(p.err_word, err);
     __syncthreads();
     finish_launch(p.ws, epoch);   // the last block out clears the abort flag and the stall settings
