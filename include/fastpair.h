@@ -276,7 +276,9 @@ const char* fp_last_error(void);
  * the look-back that needs it polls it `spin_limit` times (1..2^20; the
  * built-in limit is 2^20 polls with back-off), then gives up; the
  * one-launch decode's first grid barrier starts with an arrival count no
- * grid reaches, so its blocks give up there in the same way.  The call
+ * grid reaches, so its blocks give up there in the same way; the
+ * one-cluster decode waits for nothing but the hardware barrier and reports
+ * the timeout at once.  The call
  * reports FP_ERR_TIMEOUT through fp_sync_status; its output is unspecified
  * but every write stays in bounds.  Both settings end with that call: the
  * next decode on the stream is normal.
@@ -526,8 +528,9 @@ fp_status fp_serve_destroy(fp_server* server);
  *                   kernel launches of one fp_decode call (2: index pass and
  *                   block-pipeline decode; 3: index pass and reduce in one
  *                   launch, tile scan, warp-tile decode; 1: the warp-tile
- *                   passes as phases of one cooperative launch, for small
- *                   columns).  Any out pointer may be NULL.
+ *                   passes as phases of one launch, cooperative or of one
+ *                   cluster, for small columns).  Any out pointer may be
+ *                   NULL.
  * fp_variant_select make variant v the one fp_decode uses for the codec in
  *                   this process (v = -1 restores the defaults: tuned ones
  *                   (fp_tune_*), else built-in ones, which depend on the

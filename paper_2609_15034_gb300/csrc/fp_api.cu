@@ -170,9 +170,31 @@ fp_status grid_for(const Variant& var, int* grid_per_wave, int* sms) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, var.kernel, var.threads, var.smem_bytes);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
         if (nb < 1) return fail(FP_ERR_CUDA, "decode variant does not fit on an SM");
+        if (var.warp_tiles == 3) {
+            // blocks of the largest cluster that fits (16 need not be portable)
+            e = cudaFuncSetAttribute(var.kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(cluster)");
+            for (nb = 16; nb > 1; nb /= 2) {
+                cudaLaunchConfig_t cfg = {};
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = (unsigned)nb;
+                at[0].val.clusterDim.y = 1;
+                at[0].val.clusterDim.z = 1;
+                cfg.gridDim = dim3((unsigned)nb);
+                cfg.blockDim = dim3(var.threads);
+                cfg.dynamicSmemBytes = var.smem_bytes;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                int clusters = 0;
+                e = cudaOccupancyMaxActiveClusters(&clusters, var.kernel, &cfg);
+                if (e == cudaSuccess && clusters >= 1) break;
+                cudaGetLastError();   // a size the device does not take
+            }
+        }
         it = di.blocks_per_sm.emplace(var.kernel, nb).first;
     }
-    *grid_per_wave = it->second * di.sms;
+    *grid_per_wave = var.warp_tiles == 3 ? it->second : it->second * di.sms;
     *sms = di.sms;
     return FP_OK;
 }
@@ -740,7 +762,7 @@ fp_status fp_variant_info(fp_codec codec, int v, uint32_t* threads, uint32_t* sl
     if (threads) *threads = (uint32_t)var->threads;
     if (slots_per_thread) *slots_per_thread = (uint32_t)var->slots_per_thread;
     if (dict_in_smem) *dict_in_smem = (uint32_t)var->dict_smem;
-    if (launches_per_call) *launches_per_call = var->warp_tiles == 2 ? 1u : var->warp_tiles ? 3u : 2u;
+    if (launches_per_call) *launches_per_call = var->warp_tiles >= 2 ? 1u : var->warp_tiles ? 3u : 2u;
     return FP_OK;
 }
 

@@ -60,8 +60,24 @@ const Variant* variant_get(int codec, int v) {
 // the dictionary's width picks between them.  FSST-12 stages its 32 KiB
 // table in shared memory at every size (16M strings: 1,134 GB/s with 32-slot
 // lanes, 1,113 with 16; 300k strings: 368 against 337 through L1).
+//
+// Below 2^17 slots (256 tiles of 512: one to a warp of 16 blocks) the whole
+// column goes to one cluster in one launch: 8.7-9.5 us a call back to back
+// against 12.5-13.4 for three launches, alone 24-26 against 27-29, for every
+// codec from 1k to 88k slots; at 146k-177k slots the cluster's 16 SMs are
+// the slower side (13.3-17.6 us against 12.8-13.4).  Split-read dictionaries
+// keep the three launches.
 int variant_default(int codec, uint64_t max_slots, int width) {
     const bool split = width != 16;
+    if (max_slots < (1ull << 17)) {
+        switch (codec) {
+            case FP_ONPAIR12: if (!split) return 12; break;
+            case FP_ONPAIR16: if (!split) return 7; break;
+            case FP_FSST8: return 6;
+            case FP_FSST12: return 4;
+            default: break;
+        }
+    }
     switch (codec) {
         case FP_ONPAIR12:
             if (max_slots >= (1ull << 23)) return split ? 6 : 8;
@@ -171,6 +187,29 @@ cudaError_t launch_decode(int codec, const Variant& var, const DecodeParams& p_i
         void* fargs[] = {(void*)&p, (void*)&xp, (void*)&agg, (void*)&ex};
         return cudaLaunchCooperativeKernel(var.kernel, dim3((unsigned)dg), dim3(var.threads), fargs, var.smem_bytes,
                                            stream);
+    }
+
+    if (var.warp_tiles == 3) {
+        // one cluster of up to `grid` blocks, four tiles to a block while there
+        // are blocks (OnPair-12, 36 tiles: 11.1 us a call; one tile to each
+        // of a block's 16 warps, on three blocks: 12.2)
+        unsigned blocks = 1;
+        while (blocks < (unsigned)grid && blocks * 4ull < L.n_tiles) blocks *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(blocks);
+        cfg.blockDim = dim3(var.threads);
+        cfg.dynamicSmemBytes = var.smem_bytes;
+        cfg.stream = stream;
+        cudaLaunchAttribute at[2];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = blocks;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 2;
+        return cudaLaunchKernelExC(&cfg, var.kernel, args);
     }
 
     // warp tiles: index pass + reduce in one launch, tile scan, decode.  Each

@@ -134,7 +134,8 @@ struct Variant {
     const void* kernel;   // the decode kernel
     int warp_tiles;       // 0: block pipeline (one launch after the index pass);
                           // 1: warp tiles (index pass + reduce, tile scan and warp decode launches);
-                          // 2: warp tiles in one cooperative launch (small columns)
+                          // 2: warp tiles in one cooperative launch (small columns);
+                          // 3: warp tiles in one launch of one cluster (small columns)
     int width;            // dictionary read width W: 16 = whole entry, 8 = split read (low plane,
                           // high plane only for tokens longer than 8 bytes; paper Sec. 3.2)
     const void* reduce;   // warp tiles: the reduce kernel (its first blocks run the index pass)

@@ -17,6 +17,7 @@ const Variant* variants_onpair12(int* n) {
         make_warp_variant<FP_ONPAIR12, 16, false, 20, 1, 8>(),    // split read from the global planes
         make_fused_variant<FP_ONPAIR12, 16, false, 16, 16>(),   // one launch (small columns)
         make_fused_variant<FP_ONPAIR12, 16, true, 16, 16>(),
+        make_cluster_variant<FP_ONPAIR12, 16, true, 16, 16>(),    // one cluster (small columns)
     };
     *n = (int)(sizeof(v) / sizeof(v[0]));
     return v;

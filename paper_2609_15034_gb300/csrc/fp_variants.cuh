@@ -2,6 +2,7 @@
 // in its own translation unit (fp_var16.cu, fp_var12.cu, fp_var8.cu,
 // fp_var12f.cu) so that they compile in parallel.
 #pragma once
+#include "fp_cluster.cuh"
 #include "fp_decoder.cuh"
 #include "fp_warp.cuh"
 
@@ -55,6 +56,21 @@ Variant make_fused_variant() {
     v.smem_bytes = (size_t)C::STAGED_BYTES + NW * sizeof(typename C::Area);
     v.kernel = (const void*)&fused_decode_kernel<CODEC, K, DSMEM, NW, W>;
     v.warp_tiles = 2;
+    v.width = W;
+    return v;
+}
+
+// Small columns: one launch of one cluster.
+template <int CODEC, int K, bool DSMEM, int NW, int W>
+Variant make_cluster_variant() {
+    typedef WarpCore<CODEC, K, DSMEM, W> C;
+    Variant v{};
+    v.threads = NW * 32;
+    v.slots_per_thread = K;
+    v.dict_smem = DSMEM ? 1 : 0;
+    v.smem_bytes = (size_t)C::STAGED_BYTES + NW * sizeof(typename C::Area);
+    v.kernel = (const void*)&cluster_decode_kernel<CODEC, K, DSMEM, NW, W>;
+    v.warp_tiles = 3;
     v.width = W;
     return v;
 }

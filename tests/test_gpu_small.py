@@ -1,12 +1,14 @@
-"""GPU parity where the launches of a call overlap with what comes before
-them: a producer kernel right before the decode; stream capture.  Decoding is
-exact: no tolerance."""
+"""GPU parity of the one-cluster decode of small columns, and of the launches
+that overlap: sizes around the line between one cluster and three launches,
+tile and block edges, escape runs that cross lanes, warps and blocks, slices,
+errors; a producer kernel right before the decode; stream capture.  Decoding
+is exact: no tolerance."""
 import numpy as np
 import pytest
 
 import oracle
 import synth
-from gpu_util import DeviceColumn, oracle_decode
+from gpu_util import DeviceColumn, assert_same, make_column, oracle_decode
 
 pytestmark = pytest.mark.gpu
 
@@ -22,6 +24,61 @@ def fp():
     yield m
     for c in CODECS:
         m.variant_select(c, -1)
+
+
+def cluster_variant(fp, codec):
+    one = [v for v in range(fp.variant_count(codec)) if fp.variant_info(codec, v)["launches_per_call"] == 1]
+    return one[-1]   # the cooperative launches come first
+
+
+@pytest.mark.parametrize("codec", CODECS)
+@pytest.mark.parametrize("n_slots", [0, 1, 255, 256, 257, 8191, 8193, 65537, 131071, 131072, 200001])
+def test_cluster_sizes(fp, codec, n_slots):
+    rng = np.random.default_rng(n_slots + codec)
+    toks = [rng.integers(0, 256, 1 + k % synth.MAX_TOKEN[codec], dtype=np.uint8).tobytes() for k in range(200)]
+    slots = rng.integers(0, len(toks), n_slots)
+    fp.variant_select(codec, cluster_variant(fp, codec))
+    try:
+        for first in (0, min(n_slots, 777)):
+            offs = np.sort(np.concatenate([[first, n_slots], rng.integers(first, n_slots + 1, n_slots // 7)]))
+            assert_same(make_column(codec, toks, slots, offs))
+    finally:
+        fp.variant_select(codec, -1)
+
+
+@pytest.mark.parametrize("run", [512, 8193, 40000, 40001])
+def test_cluster_escape_runs(fp, run):
+    """0xFF slots over whole lanes, warps and blocks: the entering state of
+    every later slot comes from before the run."""
+    rng = np.random.default_rng(run)
+    slots = np.concatenate([rng.integers(0, 255, 301), np.full(run, 255), rng.integers(0, 255, 20000), [7]])
+    col = make_column(synth.FSST8, [bytes([k]) * (1 + k % 8) for k in range(255)], slots, [0, len(slots)])
+    fp.variant_select(synth.FSST8, cluster_variant(fp, synth.FSST8))
+    try:
+        assert_same(col)
+    finally:
+        fp.variant_select(synth.FSST8, -1)
+
+
+@pytest.mark.parametrize("codec", CODECS)
+def test_cluster_errors(fp, codec):
+    col = synth.column(codec, 5, 900)
+    dc = DeviceColumn(col)
+    ref = oracle_decode(col)
+    fp.variant_select(codec, cluster_variant(fp, codec))
+    try:
+        st, _, _, guard_ok, _ = dc.decode(capacity=ref.total - 1)
+        assert st == fp.ERR_CAPACITY and guard_ok
+        few = make_column(codec, [b"ab", b"c"], [0, 1, 0, 2, 1], [0, 2, 5])
+        st, _, _, guard_ok, _ = DeviceColumn(few).decode(capacity=64)
+        assert st == fp.ERR_CORRUPT and guard_ok
+        # the stall hook: nothing waits here, the call reports it and the next one is normal
+        assert fp.debug_stall_next(64) == fp.OK
+        st, _, _, guard_ok, _ = dc.decode(capacity=ref.total)
+        assert st == fp.ERR_TIMEOUT and guard_ok
+        assert_same(col, dc)
+    finally:
+        fp.variant_select(codec, -1)
 
 
 @pytest.mark.parametrize("codec", CODECS)
