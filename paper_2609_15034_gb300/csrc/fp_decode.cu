@@ -166,7 +166,7 @@ cudaError_t launch_decode(int codec, const Variant& var, const DecodeParams& p_i
     const uint64_t tile = variant_tile(var);
     const uint64_t nb = (uint64_t)p.n_strings + 1;
     uint64_t ib = (nb + 256 * kIdxGroup - 1) / (256 * kIdxGroup);
-    if (ib > (uint64_t)sms * 2) ib = (uint64_t)sms * 2;   // two index blocks per SM (an A/B: 8 per SM was 0.4 % slower)
+    if (ib > (uint64_t)sms * 2) ib = (uint64_t)sms * 2;   // two index blocks per SM
     cudaError_t e;
     void* args[] = {(void*)&p};
     if (!var.warp_tiles) {
@@ -217,10 +217,9 @@ cudaError_t launch_decode(int codec, const Variant& var, const DecodeParams& p_i
     // before it reads that launch's results.
     const uint64_t n_wt_max = L.n_tiles;   // upper bound; the kernels compute the true count
     uint64_t rg = (n_wt_max + 7) / 8;
-    const uint64_t rg_cap = (uint64_t)sms * 8;
-    if (rg > rg_cap) rg = rg_cap;
+    if (rg > (uint64_t)sms * 8) rg = (uint64_t)sms * 8;
     u32 ib32 = (u32)ib;
-    void* rargs[] = {(void*)&p, (void*)&xp, (void*)&agg, (void*)&ib32};
+    void* rargs[] = {(void*)&p, (void*)&agg, (void*)&ib32};
     e = launch_after(var.reduce, dim3((unsigned)(rg + ib)), dim3(256), rargs, 0, stream);
     if (e != cudaSuccess) return e;
     uint64_t sg = n_wt_max / kScanTile + 1;

@@ -97,6 +97,11 @@ __device__ __forceinline__ u32 in_order(const u32* a) {
     asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(a));
     return v;
 }
+__device__ __forceinline__ uint4 in_order4(const u32* a) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(a));
+    return v;
+}
 // The same past L1 (words that other SMs wrote in this launch or the one before).
 __device__ __forceinline__ u32 in_order_l2(const u32* a) {
     u32 v;

@@ -139,7 +139,7 @@ struct Variant {
     int width;            // dictionary read width W: 16 = whole entry, 8 = split read (low plane,
                           // high plane only for tokens longer than 8 bytes; paper Sec. 3.2)
     const void* reduce;   // warp tiles: the reduce kernel (its first blocks run the index pass)
-    const void* scan;     // warp tiles: the tile scan kernel
+    const void* scan;     // warp tiles: the tile scan kernel 
 };
 
 // Variant tables (fp_decode.cu).

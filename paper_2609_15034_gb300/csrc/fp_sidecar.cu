@@ -99,11 +99,10 @@ struct Path {
     static const void* decode_kernel() {
         return (const void*)&warp_decode_kernel<CODEC, K, DSMEM, kSidecarWarps, 1, W, false, true, false>;
     }
-    // Index pass in blocks [0, ib), reduce in the next rg blocks (rg = 0: index only).
-    static cudaError_t index_reduce(const DecodeParams& p, Extent* xp, u64* agg, uint64_t ib, uint64_t rg,
-                                    cudaStream_t s) {
+    // Index pass in blocks [0, ib), reduce in the next rg blocks.
+    static cudaError_t index_reduce(const DecodeParams& p, u64* agg, uint64_t ib, uint64_t rg, cudaStream_t s) {
         u32 ib32 = (u32)ib;
-        void* args[] = {(void*)&p, (void*)&xp, (void*)&agg, (void*)&ib32};
+        void* args[] = {(void*)&p, (void*)&agg, (void*)&ib32};
         return cudaLaunchKernel((const void*)&reduce_kernel<CODEC, K, DSMEM>, dim3((unsigned)(ib + rg)), dim3(256),
                                 args, 0, s);
     }
@@ -201,11 +200,10 @@ uint64_t index_blocks(uint32_t n_strings, int sms) {
 template <int CODEC>
 cudaError_t build_launches(const DecodeParams& p, char* scratch, const Layout& L, u64* ex, int sms, cudaStream_t s) {
     typedef Path<CODEC> P;
-    Extent* xp = reinterpret_cast<Extent*>(scratch + L.o_extent);
     u64* agg = reinterpret_cast<u64*>(scratch + L.o_agg);
     uint64_t rg = (L.n_tiles + 7) / 8;
     if (rg > (uint64_t)sms * 8) rg = (uint64_t)sms * 8;
-    cudaError_t e = P::index_reduce(p, xp, agg, index_blocks(p.n_strings, sms), rg, s);
+    cudaError_t e = P::index_reduce(p, agg, index_blocks(p.n_strings, sms), rg, s);
     if (e != cudaSuccess) return e;
     uint64_t sg = L.n_tiles / kScanTile + 1;
     if (sg > (uint64_t)sms * 2) sg = (uint64_t)sms * 2;
@@ -216,8 +214,8 @@ template <int CODEC>
 cudaError_t decode_launches(const DecodeParams& p, char* scratch, const Layout& L, const u64* sidecar, int sms,
                             cudaStream_t s) {
     typedef Path<CODEC> P;
-    Extent* xp = reinterpret_cast<Extent*>(scratch + L.o_extent);
-    cudaError_t e = P::index_reduce(p, xp, nullptr, index_blocks(p.n_strings, sms), 0, s);
+    index_only_kernel<<<(unsigned)index_blocks(p.n_strings, sms), 256, 0, s>>>(p, tile_slots(CODEC));
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     sidecar_check_kernel<<<1, 32, 0, s>>>(sidecar, p.capacity, p.err_word);
     e = cudaGetLastError();

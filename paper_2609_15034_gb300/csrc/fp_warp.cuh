@@ -1,12 +1,12 @@
 // Warp-tile decoder: the column is cut into warp tiles of 32*K code slots,
 // and a decode runs in three launches:
 //
-//   reduce_kernel   its first blocks run the index pass (the first string
-//                   boundary of every warp tile); in the others each warp
-//                   computes the scan element of a warp tile (its decoded
-//                   bytes; for FSST-8 the two-state element of the escape
-//                   parity) and stores it: fully parallel, the code stream
-//                   is read once;
+//   reduce_kernel   its first blocks
+//                   run the index pass (the first string boundary of every
+//                   warp tile); in the others each warp computes the scan
+//                   element of a warp tile (its decoded bytes; for FSST-8
+//                   the two-state element of the escape parity) and stores
+//                   it: fully parallel, the code stream is read once;
 //   tiles_scan_kernel  single-pass exclusive scan of the warp-tile elements
 //                   (blocks of 2,048 elements, decoupled look-back across
 //                   blocks): every warp tile's output offset and entering
@@ -974,11 +974,79 @@ struct WarpCore {
 };
 
 // ---------------------------------------------------------------------------
+// Index pass by warps: warp w of nw takes chunks of 256 boundaries, eight
+// consecutive ones to a lane (two 16-byte loads), the next chunk's loads in
+// flight.  Results and checks as index_groups(), which takes what is out of
+// the ordinary here: the first and last chunk, boundaries that decrease or
+// reach the column's ends.  About 15 instructions per 32 boundaries against
+// 60 with a boundary to a lane.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void index_by_warps(const DecodeParams& p, const Extent& x, u32 tile_log2, u32 w, u32 nw,
+                                               u32* first) {
+    constexpr u32 CH = 32 * kIdxGroup;
+    static_assert(kIdxGroup == 8, "two 16-byte loads");
+    const u32 lane = threadIdx.x & 31u;
+    const u32* a = p.code_offsets;
+    const u32 n = p.n_strings;             // the last boundary
+    const u32 chunks = n / CH + 1u;        // boundaries 0 .. n
+    const bool aligned = (reinterpret_cast<uintptr_t>(a) & 15u) == 0u;
+    const u32 cb = (u32)x.c_begin, ce = (u32)x.c_end;
+    u32* const f = first - x.first_tile;   // indexed by slot position >> tile_log2
+    u32 err = x.bad ? ERRB_CORRUPT : 0u;
+    u32 v[kIdxGroup], before = 0u;
+    auto load = [&](u32 c) {
+        const u32 i0 = c * CH + lane * kIdxGroup;
+        if (aligned && c + 1u < chunks) {
+            const uint4 lo = in_order4(a + i0), hi = in_order4(a + i0 + 4);
+            v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w;
+            v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
+        } else {
+#pragma unroll
+            for (u32 k = 0; k < kIdxGroup; ++k) v[k] = in_order(a + (n - i0 >= k && i0 <= n ? i0 + k : n));
+        }
+        before = c > 0u ? in_order(a + c * CH - 1u) : 0u;
+    };
+    if (w < chunks) load(w);
+    for (u32 c = w; c < chunks; c += nw) {
+        u32 cur[kIdxGroup];
+#pragma unroll
+        for (int k = 0; k < kIdxGroup; ++k) cur[k] = v[k];
+        u32 prev = __shfl_up_sync(0xffffffffu, cur[kIdxGroup - 1], 1);
+        if (lane == 0u) prev = before;
+        if (chunks - c > nw) load(c + nw);
+        const u32 i0 = c * CH + lane * kIdxGroup;
+        bool plain = prev >= cb && cur[kIdxGroup - 1] < ce && prev <= cur[0];
+#pragma unroll
+        for (int k = 1; k < kIdxGroup; ++k) plain &= cur[k - 1] <= cur[k];
+        if (c > 0u && c + 1u < chunks && __all_sync(0xffffffffu, plain)) {
+            u32 t = prev >> tile_log2;
+#pragma unroll
+            for (int k = 0; k < kIdxGroup; ++k) {
+                const u32 u = cur[k] >> tile_log2;
+                for (; t < u; ++t) f[t + 1u] = i0 + k;   // tiles that begin between the two boundaries
+            }
+        } else {
+#pragma unroll
+            for (u32 k = 0; k < kIdxGroup; ++k) {
+                if (i0 <= n && n - i0 >= k) index_one(x, tile_log2, (u64)n + 1, (u64)i0 + k, cur[k], prev, first, err);
+                prev = cur[k];
+            }
+        }
+    }
+    if (err) atomicOr(p.err_word, err);
+}
+
+// The index pass alone (a stored table replaces the other passes).
+__global__ void __launch_bounds__(256) index_only_kernel(const DecodeParams p, u32 tile) {
+    index_by_warps(p, column_extent(p, tile), (u32)(__ffs((int)tile) - 1), blockIdx.x * 8u + (threadIdx.x >> 5),
+                   gridDim.x * 8u, const_cast<u32*>(p.first));
+}
+
+// ---------------------------------------------------------------------------
 // Pass 1: warp-tile elements.
 // ---------------------------------------------------------------------------
 // Blocks [0, index_blocks) run the index pass (first string of every warp
-// tile; block 0 also stores the column's extent for the later passes), the
-// others the reduce: the two overlap in one launch.
+// tile), the others the reduce: the two overlap in one launch.
 // Reduce shape per codec, from an A/B on GB300 (10M-16M strings): rounds of
 // kReduceU tiles in flight, kReduceMinB blocks of 256 threads per SM.
 // OnPair-12: 2 x 4 (1,515 GB/s per call against 1,498 at 2 x 3); FSST-8,
@@ -991,7 +1059,7 @@ struct ReduceShape {
 };
 
 template <int CODEC, int K, bool DSMEM, bool PACKED = false>
-__global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kernel(const DecodeParams pp, Extent* xp,
+__global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kernel(const DecodeParams pp,
                                                                                   u64* agg, u32 index_blocks) {
     typedef WarpCore<CODEC, K, DSMEM, WarpCore<CODEC, K, DSMEM>::TOK8 ? 8 : 16, PACKED> C;
     __shared__ __align__(16) uint8_t s_lens[DSMEM ? C::LENS_BYTES : 16];
@@ -1006,11 +1074,8 @@ __global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kerne
     p.codes = after_wait(pp.codes);
     grid_release();   // the next launch may be scheduled as these blocks retire (it waits for their results)
     if (blockIdx.x < index_blocks) {
-        const Extent x = column_extent(p, C::TILE);
-        if (blockIdx.x == 0 && threadIdx.x == 0) *xp = x;
-        index_groups(p, x, (u32)(__ffs(C::TILE) - 1), 0, (u64)p.n_strings + 1,
-                     (u64)blockIdx.x * blockDim.x + threadIdx.x, (u64)index_blocks * blockDim.x,
-                     const_cast<u32*>(p.first));
+        index_by_warps(p, column_extent(p, C::TILE), (u32)(__ffs(C::TILE) - 1), blockIdx.x * 8u + (threadIdx.x >> 5),
+                       index_blocks * 8u, const_cast<u32*>(p.first));
         return;
     }
     if (DSMEM) __syncthreads();
@@ -1231,8 +1296,8 @@ __device__ __forceinline__ void renew_launch(WsHeader* ws) {
 // tag, the column's extent) is fetched while the reduce still runs: on a
 // small column the scan is a chain of global round trips.
 template <bool FSST>
-__global__ void __launch_bounds__(256) tiles_scan_kernel(const DecodeParams p, u32 tile, const u64* agg, u64* ex,
-                                                         unsigned long long* status) {
+__global__ void __launch_bounds__(256, 4) tiles_scan_kernel(const DecodeParams p, u32 tile, const u64* agg, u64* ex,
+                                                            unsigned long long* status) {
     __shared__ ScanShared sh;
     WsHeader* ws = p.ws;
     grid_release();   // the decode may start launching (its blocks stage the dictionary, then wait)
