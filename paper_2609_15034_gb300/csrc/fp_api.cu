@@ -166,6 +166,11 @@ fp_status grid_for(const Variant& var, int* grid_per_wave, int* sms) {
     if (it == di.blocks_per_sm.end()) {
         e = cudaFuncSetAttribute(var.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)var.smem_bytes);
         if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+        if (var.reduce_large) {
+            e = cudaFuncSetAttribute(var.reduce_large, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)var.reduce_large_smem);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(reduce)");
+        }
         int nb = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, var.kernel, var.threads, var.smem_bytes);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");

@@ -4,6 +4,7 @@
 // decode, or index pass and reduce in one grid + tile scan + warp-tile
 // decode).
 #include "fp_decoder.cuh"
+#include "fp_reduce.cuh"
 #include "fp_warp.cuh"
 
 namespace fp {
@@ -216,11 +217,14 @@ cudaError_t launch_decode(int codec, const Variant& var, const DecodeParams& p_i
     // may start while the launch before it finishes and waits in the kernel
     // before it reads that launch's results.
     const uint64_t n_wt_max = L.n_tiles;   // upper bound; the kernels compute the true count
-    uint64_t rg = (n_wt_max + 7) / 8;
-    if (rg > (uint64_t)sms * 8) rg = (uint64_t)sms * 8;
-    u32 ib32 = (u32)ib;
-    void* rargs[] = {(void*)&p, (void*)&agg, (void*)&ib32};
-    e = launch_after(var.reduce, dim3((unsigned)(rg + ib)), dim3(256), rargs, 0, stream);
+    const bool large = var.reduce_large && max_slots >= var.reduce_large_slots;
+    const uint64_t rw = large ? var.reduce_large_threads / 32 : 8, rg_cap = (uint64_t)sms * (large ? 1 : 8);
+    uint64_t rg = (n_wt_max + rw - 1) / rw;
+    if (rg > rg_cap) rg = rg_cap;
+    u32 index = large ? reduce_index_warps(nb, rg) : (u32)ib;   // warps of every block, or blocks
+    void* rargs[] = {(void*)&p, (void*)&agg, (void*)&index};
+    if (large) e = launch_after(var.reduce_large, dim3((unsigned)rg), dim3(var.reduce_large_threads), rargs, var.reduce_large_smem, stream);
+    else e = launch_after(var.reduce, dim3((unsigned)(rg + ib)), dim3(256), rargs, 0, stream);
     if (e != cudaSuccess) return e;
     uint64_t sg = n_wt_max / kScanTile + 1;
     if (sg > (uint64_t)sms * 2) sg = (uint64_t)sms * 2;

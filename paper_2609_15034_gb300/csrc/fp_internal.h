@@ -139,6 +139,10 @@ struct Variant {
     int width;            // dictionary read width W: 16 = whole entry, 8 = split read (low plane,
                           // high plane only for tokens longer than 8 bytes; paper Sec. 3.2)
     const void* reduce;   // warp tiles: the reduce kernel (its first blocks run the index pass)
+    const void* reduce_large;      // the one for buffers of at least reduce_large_slots slots, or null
+    uint64_t reduce_large_slots;
+    int reduce_large_threads;
+    size_t reduce_large_smem;
     const void* scan;     // warp tiles: the tile scan kernel 
 };
 

@@ -4,6 +4,7 @@
 #pragma once
 #include "fp_cluster.cuh"
 #include "fp_decoder.cuh"
+#include "fp_reduce.cuh"
 #include "fp_warp.cuh"
 
 namespace fp {
@@ -40,6 +41,12 @@ Variant make_warp_variant() {
     v.kernel = (const void*)&warp_decode_kernel<CODEC, K, DSMEM, NW, MINB, W, false, LSMEM>;
     v.warp_tiles = 1;
     v.reduce = (const void*)&reduce_kernel<CODEC, K, DSMEM>;
+    if constexpr (LargeReduce<CODEC, K>::slots != 0) {
+        v.reduce_large = (const void*)&length_reduce_kernel<CODEC, K>;
+        v.reduce_large_slots = LargeReduce<CODEC, K>::slots;
+        v.reduce_large_threads = LargeReduce<CODEC, K>::threads;
+        v.reduce_large_smem = LengthTable<CODEC, K>::BYTES;
+    }
     v.scan = (const void*)&tiles_scan_kernel<CODEC == FP_FSST8>;
     v.width = W;
     return v;

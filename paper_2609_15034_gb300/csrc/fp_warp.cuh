@@ -1,7 +1,7 @@
 // Warp-tile decoder: the column is cut into warp tiles of 32*K code slots,
 // and a decode runs in three launches:
 //
-//   reduce_kernel   its first blocks
+//   reduce_kernel (or length_reduce_kernel, fp_reduce.cuh)  its first blocks
 //                   run the index pass (the first string boundary of every
 //                   warp tile); in the others each warp computes the scan
 //                   element of a warp tile (its decoded bytes; for FSST-8
@@ -1046,7 +1046,8 @@ __global__ void __launch_bounds__(256) index_only_kernel(const DecodeParams p, u
 // Pass 1: warp-tile elements.
 // ---------------------------------------------------------------------------
 // Blocks [0, index_blocks) run the index pass (first string of every warp
-// tile), the others the reduce: the two overlap in one launch.
+// tile), the others the reduce: the two overlap in one launch.  Large FSST-8
+// and OnPair-16 columns take length_reduce_kernel (fp_reduce.cuh) instead.
 // Reduce shape per codec, from an A/B on GB300 (10M-16M strings): rounds of
 // kReduceU tiles in flight, kReduceMinB blocks of 256 threads per SM.
 // OnPair-12: 2 x 4 (1,515 GB/s per call against 1,498 at 2 x 3); FSST-8,
