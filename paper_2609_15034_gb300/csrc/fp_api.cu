@@ -353,7 +353,7 @@ fp_status run_rows(fp_codec codec, const fp_dict* dict, const void* d_codes, uin
     char* scratch = static_cast<char*>(w->d_mem) + kWsHeaderBytes;
     char* rows = scratch + dec_bytes;
     WsHeader* ws = static_cast<WsHeader*>(w->d_mem);
-    const RowsArgs a{static_cast<const uint8_t*>(d_codes), max_slots_of(codec, codes_bytes), d_code_offsets,
+    const RowsArgs a{static_cast<const uint8_t*>(d_codes), codes_bytes, max_slots_of(codec, codes_bytes), d_code_offsets,
                      n_strings, d_row_ids, n_rows};
     cudaError_t e = launch_rows_gather(codec, a, slots, true, rows, RL, ws, sms, stream);
     if (e != cudaSuccess) return cuda_fail(e, "row gather launch");
@@ -498,7 +498,7 @@ fp_status fp_rows_size(fp_codec codec, const fp_dict* dict, const void* d_codes,
     int dev_sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, dict->device);
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
-    const RowsArgs a{static_cast<const uint8_t*>(d_codes), max_slots_of(codec, codes_bytes), d_code_offsets,
+    const RowsArgs a{static_cast<const uint8_t*>(d_codes), codes_bytes, max_slots_of(codec, codes_bytes), d_code_offsets,
                      n_strings, d_row_ids, n_rows};
     e = launch_rows_gather(codec, a, ~0ull, false, static_cast<char*>(w->d_mem) + kWsHeaderBytes, RL0,
                            static_cast<WsHeader*>(w->d_mem), dev_sms, stream);

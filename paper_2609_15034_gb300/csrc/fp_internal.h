@@ -175,6 +175,7 @@ cudaError_t launch_plain(int codec, const DecodeParams& p, uint32_t* d_scratch, 
 // codes are gathered.
 struct RowsArgs {
     const uint8_t* codes;          // the column's stored code buffer
+    uint64_t codes_bytes;
     uint64_t max_slots;            // whole slots in it
     const uint32_t* code_offsets;  // n_strings + 1
     uint32_t n_strings;
@@ -182,16 +183,17 @@ struct RowsArgs {
     uint32_t n_rows;
 };
 // Scratch of a selective decode (after the decode's own scratch): the
-// virtual code offsets v[0 .. n_rows], the scan's block sums, the gathered
-// stream (codes_bytes of it are handed to the decode).
+// virtual code offsets v[0 .. n_rows], each row's first stored slot, the scan's
+// block sums, the row each gather chunk begins in, the gathered stream
+// (codes_bytes of it are handed to the decode).
 struct RowsLayout {
-    size_t o_v, o_sums, o_codes, bytes;
+    size_t o_v, o_src, o_sums, o_row_of, o_codes, bytes;
     uint64_t codes_bytes;
 };
 RowsLayout rows_layout(int codec, uint32_t n_rows, uint64_t selected_slots);
 // Row lengths, their scan into v (ws->rows_slots gets the total; more than
 // selected_slots sets ERRB_CAPACITY) and, with `gather`, the gather of at
-// most selected_slots codes: three or four launches.
+// most selected_slots codes: two or three launches, one more for many rows.
 cudaError_t launch_rows_gather(int codec, const RowsArgs& a, uint64_t selected_slots, bool gather, void* scratch,
                                const RowsLayout& L, WsHeader* ws, int sms, cudaStream_t stream);
 size_t plain_scratch_words(uint32_t n_strings);

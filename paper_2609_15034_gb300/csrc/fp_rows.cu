@@ -3,11 +3,13 @@
 //
 // The selected rows' code slots are laid out one after another in a virtual
 // slot space: row k occupies virtual slots [v[k], v[k+1]), v being the
-// exclusive scan of the rows' slot counts.  Three launches build v (the
-// per-block sums of the row lengths, the scan of those sums, the per-block
-// exclusive offsets), a fourth gathers the selected codes into one
-// contiguous stored stream (each thread writes whole aligned words of it), and
-// fp_decode's kernels then decode that stream with v as its code_offsets.
+// exclusive scan of the rows' slot counts.  Two launches build v and, for every
+// 32 groups of virtual slots, the row they begin in (per-block sums of the row
+// lengths, then the offsets, each block adding up the sums before it; a
+// selection of more than 8 M rows has the sums scanned by a launch between
+// them); the next gathers the selected codes into one contiguous stored
+// stream (each thread writes whole aligned words of it), and fp_decode's
+// kernels then decode that stream with v as its code_offsets.
 #include <cstddef>
 
 #include "fp_decoder.cuh"
@@ -18,36 +20,45 @@ namespace {
 constexpr int kRowBlock = 256;
 constexpr int kRowItems = 2048;   // rows per scan block (8 per thread)
 constexpr int kRowPer = kRowItems / kRowBlock;
-
-// Slot count of selected row k (0, with ERRB_CORRUPT, for a bad row).
-__device__ __forceinline__ u32 row_len(const RowsArgs& a, u32 k, u32& err) {
-    const u32 id = __ldg(a.row_ids + k);
-    if (id >= a.n_strings) {
-        err |= ERRB_CORRUPT;
-        return 0u;
-    }
-    const u32 b = __ldg(a.code_offsets + id), e = __ldg(a.code_offsets + id + 1);
-    if (e < b || (u64)e > a.max_slots) {
-        err |= ERRB_CORRUPT;
-        return 0u;
-    }
-    return e - b;
-}
+constexpr u32 kRowDirect = 4096;  // blocks up to which every block adds up the sums before it
+// Virtual slots of a gather thread, and of a warp (a chunk).
+constexpr int row_group(int codec) { return codec == FP_FSST8 ? 16 : 8; }
+constexpr int row_chunk(int codec) { return 32 * row_group(codec); }
 
 // Pass 1: each block sums the slot counts of its kRowItems rows and stores
-// the counts in v[] (the next pass turns them into offsets in place).
-__global__ void __launch_bounds__(kRowBlock) rows_sums_kernel(const RowsArgs a, u32* v, u64* block_sums,
+// the counts in v[] (the next pass turns them into offsets in place) and
+// each row's first slot in src[].  A bad row (its id, or its offsets) counts 0
+// slots and sets ERRB_CORRUPT.  The offsets are read from random places: a
+// thread's eight row ids, then its sixteen offsets are in flight together,
+// with no branch between them (500k rows: 14 us with one).
+__global__ void __launch_bounds__(kRowBlock) rows_sums_kernel(const RowsArgs a, u32* v, u32* src, u64* block_sums,
                                                             unsigned* err_word) {
     __shared__ u64 red[kRowBlock / 32];
-    const u64 base = (u64)blockIdx.x * kRowItems + (u64)threadIdx.x * kRowPer;
+    grid_release();
+    const u64 base = (u64)blockIdx.x * kRowItems + threadIdx.x;
     u32 err = 0;
     u64 s = 0;
+    u32 id[kRowPer], b[kRowPer], e[kRowPer];
 #pragma unroll
     for (int k = 0; k < kRowPer; ++k) {
-        const u64 r = base + k;
+        const u64 r = base + k * kRowBlock;
+        id[k] = r < a.n_rows ? __ldg(a.row_ids + r) : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < kRowPer; ++k) {
+        const u32 i = id[k] < a.n_strings ? id[k] : 0u;
+        b[k] = __ldg(a.code_offsets + i);
+        e[k] = __ldg(a.code_offsets + i + (a.n_strings ? 1u : 0u));
+    }
+#pragma unroll
+    for (int k = 0; k < kRowPer; ++k) {
+        const u64 r = base + k * kRowBlock;
+        const bool bad = id[k] >= a.n_strings || e[k] < b[k] || (u64)e[k] > a.max_slots;
+        const u32 L = bad ? 0u : e[k] - b[k];
         if (r < a.n_rows) {
-            const u32 L = row_len(a, (u32)r, err);
+            if (bad) err |= ERRB_CORRUPT;
             v[r] = L;
+            src[r] = b[k];
             s += L;
         }
     }
@@ -63,13 +74,14 @@ __global__ void __launch_bounds__(kRowBlock) rows_sums_kernel(const RowsArgs a, 
     if (err) atomicOr(err_word, err);
 }
 
-// Pass 2 (one block): exclusive scan of the block sums; the total goes to
-// ws->rows_slots and must fit the bound (and 32-bit offsets).
-__global__ void __launch_bounds__(kRowBlock) rows_scan_sums_kernel(u64* block_sums, u32 nb, u64 bound, WsHeader* ws) {
+// Between the passes, for many rows (one block): exclusive scan of the block sums.
+__global__ void __launch_bounds__(kRowBlock) rows_scan_sums_kernel(u64* block_sums, u32 nb) {
     __shared__ u64 wsum[kRowBlock / 32];
     __shared__ u64 carry_s;
     const u32 lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) carry_s = 0;
+    grid_wait();
+    grid_release();
     __syncthreads();
     for (u32 base = 0; base < nb; base += kRowBlock) {
         const u32 i = base + threadIdx.x;
@@ -93,18 +105,20 @@ __global__ void __launch_bounds__(kRowBlock) rows_scan_sums_kernel(u64* block_su
         if (threadIdx.x == 0) carry_s = carry + tot;
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        const u64 total = carry_s;
-        ws->rows_slots = total;
-        if (total > bound || total > 0xffffffffull) atomicOr(&ws->status, ERRB_CAPACITY);
-    }
 }
 
-// Pass 3: v[k] = slots of the rows before k (in place), v[n_rows] = total.
-__global__ void __launch_bounds__(kRowBlock) rows_offsets_kernel(const RowsArgs a, u32* v, const u64* block_sums) {
-    __shared__ u64 wsum[kRowBlock / 32];
+// Pass 2: v[k] = slots of the rows before k (in place), v[n_rows] = total,
+// and row_of[c] = the row that holds virtual slot c * chunk.  The last block
+// checks the total against the bound (and 32-bit offsets).  `scanned`: the
+// block sums are offsets already.
+__global__ void __launch_bounds__(kRowBlock) rows_offsets_kernel(const RowsArgs a, u32* v, const u64* block_sums,
+                                                               u32 scanned, u32* row_of, u32 chunk_log2, u64 bound,
+                                                               WsHeader* ws) {
+    __shared__ u64 wsum[kRowBlock / 32], wbefore[kRowBlock / 32];
     const u32 lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const u64 base = (u64)blockIdx.x * kRowItems + (u64)threadIdx.x * kRowPer;
+    grid_wait();
+    grid_release();
     u32 len[kRowPer];
     u64 s = 0;
 #pragma unroll
@@ -113,98 +127,164 @@ __global__ void __launch_bounds__(kRowBlock) rows_offsets_kernel(const RowsArgs 
         len[k] = r < a.n_rows ? v[r] : 0u;
         s += len[k];
     }
+    u64 prior = 0;   // this thread's share of the blocks before
+    if (!scanned)
+        for (u32 i = threadIdx.x; i < blockIdx.x; i += kRowBlock) prior += block_sums[i];
     u64 inc = s;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const u64 y = __shfl_up_sync(0xffffffffu, inc, d);
         if (lane >= (u32)d) inc += y;
     }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) prior += __shfl_down_sync(0xffffffffu, prior, d);
     if (lane == 31) wsum[warp] = inc;
+    if (lane == 0) wbefore[warp] = prior;
     __syncthreads();
-    u64 before = 0;
-    for (u32 w = 0; w < warp; ++w) before += wsum[w];
-    u64 o = block_sums[blockIdx.x] + before + inc - s;
+    u64 o = scanned ? block_sums[blockIdx.x] : 0;
+#pragma unroll
+    for (u32 w = 0; w < kRowBlock / 32; ++w) {
+        o += scanned ? 0 : wbefore[w];
+        if (w < warp) o += wsum[w];
+    }
+    o += inc - s;
 #pragma unroll
     for (int k = 0; k < kRowPer; ++k) {
         const u64 r = base + k;
-        if (r <= a.n_rows) v[r] = (u32)o;   // r == n_rows: the total (32 bits; larger totals were flagged)
+        if (r <= a.n_rows) v[r] = (u32)o;   // r == n_rows: the total (32 bits; larger totals are flagged)
+        if (r == a.n_rows) {
+            ws->rows_slots = o;
+            if (o > bound || o > 0xffffffffull) atomicOr(&ws->status, ERRB_CAPACITY);
+        }
+        const u64 end = o + len[k] < bound ? o + len[k] : bound;
+        if (row_of)
+            for (u64 c = (o + (1u << chunk_log2) - 1) >> chunk_log2; (c << chunk_log2) < end; ++c) row_of[c] = (u32)r;
         o += len[k];
     }
 }
 
-// Code in physical slot q of the stored stream.
+// Bits below b of a word (b may lie outside 0 .. 32).
+__device__ __forceinline__ u32 bits_below(int b) { return b <= 0 ? 0u : (b >= 32 ? 0xffffffffu : (1u << b) - 1u); }
+
+// Pass 3: gather.  A warp writes a chunk of 32 groups of G virtual slots of
+// the compacted stream, a lane one group as whole words: 8 slots of 16 or 12
+// bits (4 or 3 words), 16 slots of 8 bits (4 words).  The rows of the chunk
+// (about 14 of 18 codes) are looked up in a window in shared memory, and a
+// row's part of a group is one window of aligned words of the stored stream
+// shifted into place: 5 or 4 word loads, where a byte or two per slot took up
+// to 16 loads and a search over all rows 20 more (1M rows of 18 12-bit codes:
+// GATHER_US).  Slots past the selected total (or the bound) are written as
+// zero and never decoded.
 template <int CODEC>
-__device__ __forceinline__ u32 read_code(const uint8_t* s, u64 q) {
-    if (CODEC == FP_ONPAIR16) return (u32)__ldg(s + 2 * q) | ((u32)__ldg(s + 2 * q + 1) << 8);
-    if (CODEC == FP_ONPAIR12 || CODEC == FP_FSST12) {
-        const u64 by = q * 3 / 2;
-        const u32 lo = __ldg(s + by), hi = __ldg(s + by + 1);
-        return (q & 1) ? ((lo >> 4) | (hi << 4)) : (lo | ((hi & 0xfu) << 8));
+__global__ void __launch_bounds__(kRowBlock) rows_gather_kernel(const RowsArgs a, const u32* v, const u32* src,
+                                                              const u32* row_of, uint8_t* out, u64 bound,
+                                                              const WsHeader* ws) {
+    constexpr int BITS = CODEC == FP_ONPAIR16 ? 16 : (CODEC == FP_FSST8 ? 8 : 12);
+    constexpr int G = CODEC == FP_FSST8 ? 16 : 8, CH = 32 * G, NW = G * BITS / 32, WIN = 64;
+    __shared__ u32 s_v[kRowBlock / 32][WIN + 1], s_src[kRowBlock / 32][WIN];
+    grid_wait();
+    grid_release();
+    const u64 total_raw = *(const volatile u64*)&ws->rows_slots;
+    // a total past 32 bits left v[] wrapped (and flagged): gather nothing
+    const u64 total64 = total_raw > 0xffffffffull ? 0 : (total_raw < bound ? total_raw : bound);
+    const u32 total = (u32)total64;
+    const u32 n_chunks = (u32)((total64 + CH - 1) / CH);
+    const u32 m = a.n_rows, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    u32* const wv = s_v[warp];
+    u32* const wsrc = s_src[warp];
+    // the stored stream as words (fewer than 2^32: slots are 32-bit), zero
+    // outside it; its last bytes make a word of their own
+    const u32* const words = reinterpret_cast<const u32*>(a.codes);
+    const u32 n_words = (u32)(a.codes_bytes / 4);
+    u32 tail = 0;
+    for (u32 q = 0; q < (u32)(a.codes_bytes & 3u); ++q) tail |= (u32)__ldg(a.codes + 4ull * n_words + q) << (8 * q);
+    auto word = [&](u32 i) { return i < n_words ? __ldg(words + i) : (i == n_words ? tail : 0u); };
+    for (u32 c = blockIdx.x * (kRowBlock / 32) + warp; c < n_chunks; c += gridDim.x * (kRowBlock / 32)) {
+        const u32 k0 = row_of[c];
+        for (u32 i = lane; i <= (u32)WIN; i += 32u) {
+            wv[i] = v[min(k0 + i, m)];
+            if (i < (u32)WIN) wsrc[i] = k0 + i < m ? src[k0 + i] : 0u;
+        }
+        __syncwarp();
+        const u32 v0 = c * (u32)CH + lane * G;
+        u32 acc[NW] = {};
+        const u32 left = v0 < total ? min(total - v0, (u32)G) : 0u;
+        u32 j = 0, i = WIN;   // i: the row in the window
+        while (j < left) {
+            // the row of slot v0 + j (non-empty, so its id passed the
+            // checks): its first virtual slot, its end, its first stored slot
+            const u32 pos = v0 + j;
+            u32 vs, ve, sb;
+            if (pos < wv[WIN]) {
+                if (j == 0u) {
+                    i = 0u;
+#pragma unroll
+                    for (u32 d = WIN / 2; d > 0; d >>= 1)
+                        if (wv[i + d] <= pos) i += d;
+                } else {
+                    do ++i;
+                    while (wv[i + 1] <= pos);
+                }
+                vs = wv[i];
+                ve = wv[i + 1];
+                sb = wsrc[i];
+            } else {
+                u32 lo = k0, hi = m;   // v[lo] <= pos < v[hi]
+                while (hi - lo > 1u) {
+                    const u32 mid = lo + (hi - lo) / 2u;
+                    if (v[mid] <= pos) lo = mid;
+                    else hi = mid;
+                }
+                vs = v[lo];
+                ve = v[lo + 1];
+                sb = src[lo];
+            }
+            // the words from the stored bit of the group's slot 0 on, as if
+            // the row began early enough and ended late enough: the rows
+            // after it overwrite the rest
+            const long long bit = (long long)BITS * ((long long)sb + v0 - vs);
+            const u32 w0 = (u32)(bit >> 5);
+            u32 x[NW + 1];
+#pragma unroll
+            for (int q = 0; q <= NW; ++q) x[q] = word(w0 + q);
+#pragma unroll
+            for (int q = 0; q < NW; ++q) {
+                const u32 keep = j ? bits_below((int)j * BITS - 32 * q) : 0u;
+                acc[q] = (acc[q] & keep) | (__funnelshift_r(x[q], x[q + 1], (u32)bit) & ~keep);
+            }
+            j = min(left, ve - v0);
+        }
+        if (left < (u32)G)
+#pragma unroll
+            for (int q = 0; q < NW; ++q) acc[q] &= bits_below((int)left * BITS - 32 * q);
+        if (left) {
+            const u64 g = (u64)c * 32u + lane;
+            if (NW == 4) {
+                reinterpret_cast<uint4*>(out)[g] = make_uint4(acc[0], acc[1], acc[2], acc[NW - 1]);
+            } else {
+                u32* w = reinterpret_cast<u32*>(out) + 3 * g;
+                w[0] = acc[0];
+                w[1] = acc[1];
+                w[2] = acc[2];
+            }
+        }
+        __syncwarp();   // the window is refilled
     }
-    return __ldg(s + q);
 }
 
-// Pass 4: gather.  Thread g writes the group of G virtual slots [G g, G g + G)
-// of the compacted stream as whole words: 8 slots of 16 or 12 bits (16 or
-// 12 bytes), 16 slots of 8 bits (16 bytes).  Slots past the selected total
-// (or the bound) are written as zero and never decoded.
-template <int CODEC>
-__global__ void __launch_bounds__(kRowBlock) rows_gather_kernel(const RowsArgs a, const u32* v, uint8_t* out,
-                                                              u64 bound, const WsHeader* ws) {
-    constexpr bool W12 = (CODEC == FP_ONPAIR12 || CODEC == FP_FSST12);
-    constexpr int G = (CODEC == FP_FSST8) ? 16 : 8;
-    const u64 total_raw = ws->rows_slots;
-    // a total past 32 bits left v[] wrapped (and flagged): gather nothing
-    const u64 total = total_raw > 0xffffffffull ? 0 : (total_raw < bound ? total_raw : bound);
-    const u64 n_groups = (total + G - 1) / G;
-    const u32 m = a.n_rows;
-    for (u64 g = (u64)blockIdx.x * blockDim.x + threadIdx.x; g < n_groups; g += (u64)gridDim.x * blockDim.x) {
-        const u64 v0 = g * G;
-        // the row holding virtual slot v0: the last k with v[k] <= v0
-        u32 lo = 0, hi = m;   // v[lo] <= v0 < v[hi] (v[m] = total > v0)
-        while (hi - lo > 1) {
-            const u32 mid = (lo + hi) >> 1;
-            if ((u64)__ldg(v + mid) <= v0) lo = mid;
-            else hi = mid;
-        }
-        // row k is non-empty (v[k] <= v0 < v[k+1]), so its id passed the checks
-        u32 k = lo, held = lo;
-        u64 row_end = __ldg(v + k + 1);
-        u64 shift = (u64)__ldg(a.code_offsets + __ldg(a.row_ids + k)) - (u64)__ldg(v + k);   // physical - virtual
-        u32 c[G];
-#pragma unroll
-        for (int j = 0; j < G; ++j) {
-            const u64 vs = v0 + j;
-            u32 code = 0;
-            if (vs < total) {
-                // skip to the row holding vs (empty rows, bad ids among them, are passed over)
-                while (vs >= row_end && k + 1 < m) row_end = __ldg(v + (++k) + 1);
-                if (vs < row_end) {
-                    if (k != held) {
-                        shift = (u64)__ldg(a.code_offsets + __ldg(a.row_ids + k)) - (u64)__ldg(v + k);
-                        held = k;
-                    }
-                    code = read_code<CODEC>(a.codes, vs + shift);
-                }
-            }
-            c[j] = code;
-        }
-        if (CODEC == FP_ONPAIR16) {
-            reinterpret_cast<uint4*>(out)[g] = make_uint4(c[0] | (c[1] << 16), c[2] | (c[3] << 16),
-                                                          c[4] | (c[5] << 16), c[6] | (c[7] << 16));
-        } else if (W12) {
-            // 8 codes, LSB-first: 96 bits = 3 words
-            u32* w = reinterpret_cast<u32*>(out) + 3 * g;
-            w[0] = c[0] | (c[1] << 12) | (c[2] << 24);
-            w[1] = (c[2] >> 8) | (c[3] << 4) | (c[4] << 16) | (c[5] << 28);
-            w[2] = (c[5] >> 4) | (c[6] << 8) | (c[7] << 20);
-        } else {
-            reinterpret_cast<uint4*>(out)[g] =
-                make_uint4(c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24), c[4] | (c[5] << 8) | (c[6] << 16) | (c[7] << 24),
-                           c[8] | (c[9] << 8) | (c[10] << 16) | (c[11] << 24),
-                           c[12] | (c[13] << 8) | (c[14] << 16) | (c[15] << 24));
-        }
-    }
+// Launch that may start while the launch before it finishes (it waits in the kernel).
+template <class... A, class... B>
+cudaError_t launch_early(void (*kernel)(A...), u32 grid, cudaStream_t stream, B... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kRowBlock);
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, (A)args...);
 }
 
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -215,10 +295,11 @@ RowsLayout rows_layout(int codec, uint32_t n_rows, uint64_t selected_slots) {
     RowsLayout L{};
     const uint64_t nb = ((uint64_t)n_rows + kRowItems - 1) / kRowItems + 1;
     L.o_v = 0;
-    L.o_sums = al256(((size_t)n_rows + 1) * sizeof(u32));
-    L.o_codes = L.o_sums + al256(nb * sizeof(u64));
-    const uint64_t G = codec == FP_FSST8 ? 16 : 8;
-    const uint64_t group_bytes = codec == FP_FSST8 ? 16 : (code_bits(codec) * 8 / 8);
+    L.o_src = al256(((size_t)n_rows + 1) * sizeof(u32));
+    L.o_sums = L.o_src + al256(((size_t)n_rows + 1) * sizeof(u32));
+    L.o_row_of = L.o_sums + al256(nb * sizeof(u64));
+    L.o_codes = L.o_row_of + al256((selected_slots / row_chunk(codec) + 1) * sizeof(u32));
+    const uint64_t G = row_group(codec), group_bytes = G * code_bits(codec) / 8;
     const uint64_t groups = (selected_slots + G - 1) / G;
     L.codes_bytes = (selected_slots * code_bits(codec) + 7) / 8;
     L.bytes = L.o_codes + al256(groups * group_bytes + 16);
@@ -229,24 +310,31 @@ cudaError_t launch_rows_gather(int codec, const RowsArgs& a, uint64_t selected_s
                                const RowsLayout& L, WsHeader* ws, int sms, cudaStream_t stream) {
     char* base = static_cast<char*>(scratch);
     u32* v = reinterpret_cast<u32*>(base + L.o_v);
+    u32* src = reinterpret_cast<u32*>(base + L.o_src);
     u64* sums = reinterpret_cast<u64*>(base + L.o_sums);
+    u32* row_of = reinterpret_cast<u32*>(base + L.o_row_of);
     uint8_t* codes = reinterpret_cast<uint8_t*>(base + L.o_codes);
     const u32 nb = (u32)((uint64_t)a.n_rows / kRowItems) + 1;   // the blocks of v[0 .. n_rows]
-    rows_sums_kernel<<<nb, kRowBlock, 0, stream>>>(a, v, sums, &ws->status);
-    rows_scan_sums_kernel<<<1, kRowBlock, 0, stream>>>(sums, nb, selected_slots, ws);
-    rows_offsets_kernel<<<nb, kRowBlock, 0, stream>>>(a, v, sums);
-    if (!gather) return cudaGetLastError();
-    const uint64_t G = codec == FP_FSST8 ? 16 : 8;
-    uint64_t grid = (selected_slots + G * kRowBlock - 1) / (G * kRowBlock);
+    rows_sums_kernel<<<nb, kRowBlock, 0, stream>>>(a, v, src, sums, &ws->status);
+    cudaError_t e = cudaGetLastError();
+    const u32 scanned = nb > kRowDirect ? 1u : 0u;
+    if (e == cudaSuccess && scanned) e = launch_early(rows_scan_sums_kernel, 1, stream, sums, nb);
+    const u32 chunk_log2 = codec == FP_FSST8 ? 9 : 8;
+    if (e == cudaSuccess)
+        e = launch_early(rows_offsets_kernel, nb, stream, a, v, sums, scanned, gather ? row_of : nullptr, chunk_log2,
+                         selected_slots, ws);
+    if (e != cudaSuccess || !gather) return e;
+    const uint64_t per_block = (uint64_t)row_chunk(codec) * (kRowBlock / 32);
+    uint64_t grid = (selected_slots + per_block - 1) / per_block;
     if (grid > (uint64_t)sms * 8) grid = (uint64_t)sms * 8;
     if (grid < 1) grid = 1;
+    const u32 g = (u32)grid;
     switch (codec) {
-        case FP_ONPAIR16: rows_gather_kernel<FP_ONPAIR16><<<(unsigned)grid, kRowBlock, 0, stream>>>(a, v, codes, selected_slots, ws); break;
-        case FP_ONPAIR12: rows_gather_kernel<FP_ONPAIR12><<<(unsigned)grid, kRowBlock, 0, stream>>>(a, v, codes, selected_slots, ws); break;
-        case FP_FSST8: rows_gather_kernel<FP_FSST8><<<(unsigned)grid, kRowBlock, 0, stream>>>(a, v, codes, selected_slots, ws); break;
-        default: rows_gather_kernel<FP_FSST12><<<(unsigned)grid, kRowBlock, 0, stream>>>(a, v, codes, selected_slots, ws); break;
+        case FP_ONPAIR16: return launch_early(rows_gather_kernel<FP_ONPAIR16>, g, stream, a, v, src, row_of, codes, selected_slots, ws);
+        case FP_ONPAIR12: return launch_early(rows_gather_kernel<FP_ONPAIR12>, g, stream, a, v, src, row_of, codes, selected_slots, ws);
+        case FP_FSST8: return launch_early(rows_gather_kernel<FP_FSST8>, g, stream, a, v, src, row_of, codes, selected_slots, ws);
+        default: return launch_early(rows_gather_kernel<FP_FSST12>, g, stream, a, v, src, row_of, codes, selected_slots, ws);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace fp
