@@ -51,64 +51,70 @@ __device__ __forceinline__ u32 ld_here(const u32* a) {
 }
 
 // A lane's run of tokens appended to the warp's staging area as aligned
-// 32-bit words: `m` bytes of the current word (at `at`) are in `c`.
+// 64-bit words: `m` bytes of the current word (at `at`) are in c0, c1.
 //
 // Words in shared memory instead of 16-byte chunks in registers: moving a
-// token to a byte offset inside a word takes five funnel shifts and four
-// selects, moving it inside a 16-byte window took about 12 selects and 8
-// funnel shifts, and that integer work bound the decode (ALU pipe 64-72 %
-// active).  OnPair-12, 36M codes: 85 -> 65 instructions per code, the decode
-// kernel 149 -> 118 us; FSST-8, 38M slots: 77 -> 54, 134 -> 100 us.  What
-// bounds it now is the shared-memory pipe (79 % of its wavefronts on
-// OnPair-12): about 10 wavefronts per 32 codes for the table reads, 10 for
-// these stores, 3 for the lengths.
+// token into a 16-byte window took about 12 selects, 8 funnel shifts and a
+// scattered 16-byte store, and that integer work bound the decode (ALU pipe
+// 64-72 % active).  Of the word sizes, 32 bits take the fewest instructions
+// (five shifts, four selects) but up to four stores a token, 64 bits two more
+// selects per word and at most two stores, one for FSST symbols.  The decode
+// kernel, 16-byte window -> 32-bit -> 64-bit words: OnPair-12, 36M codes 149 ->
+// 118 -> 110 us; FSST-8, 38M slots 134 -> 93 -> 92; FSST-12, 33M codes 110 -> 72
+// -> 70.  What bounds it now is the shared-memory pipe (84 % of its wavefronts
+// on OnPair-12: about 10 per 32 codes for the table reads, 8 for these
+// stores, 3 for the lengths), with the ALU pipe at 66 %.
 struct StageWriter {
-    u32* at;
-    u32 m, c;
+    u64* at;
+    u32 m, c0, c1;
 
     // Continue at staging byte `pos`; a word begun by the lanes before is
     // completed here with their bytes zero, and they add theirs by
     // finish().
     __device__ __forceinline__ void begin(u32* stage, u32 pos) {
-        at = stage + (pos >> 2);
-        m = pos & 3u;
-        c = 0u;
+        at = reinterpret_cast<u64*>(stage) + (pos >> 3);
+        m = pos & 7u;
+        c0 = c1 = 0u;
     }
     // Append a token of up to 16 bytes (zero past its length).
     __device__ __forceinline__ void put(const uint4 t, u32 len) {
         const u32 sh = m * 8u;
-        const u32 s0 = c | __funnelshift_l(0u, t.x, sh), s1 = __funnelshift_l(t.x, t.y, sh),
-                  s2 = __funnelshift_l(t.y, t.z, sh), s3 = __funnelshift_l(t.z, t.w, sh),
-                  s4 = __funnelshift_l(t.w, 0u, sh);
+        const bool q = (m & 4u) != 0u;
+        const u32 y0 = __funnelshift_l(0u, t.x, sh), y1 = __funnelshift_l(t.x, t.y, sh),
+                  y2 = __funnelshift_l(t.y, t.z, sh), y3 = __funnelshift_l(t.z, t.w, sh),
+                  y4 = __funnelshift_l(t.w, 0u, sh);
+        const u32 z0 = c0 | (q ? 0u : y0), z1 = c1 | (q ? y0 : y1), z2 = q ? y1 : y2, z3 = q ? y2 : y3,
+                  z4 = q ? y3 : y4, z5 = q ? y4 : 0u;
         const u32 e = m + len;
-        if (e >= 4u) at[0] = s0;
-        if (e >= 8u) at[1] = s1;
-        if (e >= 12u) at[2] = s2;
-        if (e >= 16u) at[3] = s3;
-        c = e >= 4u ? s1 : s0;
-        c = e >= 8u ? s2 : c;
-        c = e >= 12u ? s3 : c;
-        c = e >= 16u ? s4 : c;
-        at += e >> 2;
-        m = e & 3u;
+        if (e >= 8u) *reinterpret_cast<uint2*>(at) = make_uint2(z0, z1);
+        if (e >= 16u) *reinterpret_cast<uint2*>(at + 1) = make_uint2(z2, z3);
+        c0 = e >= 8u ? z2 : z0;
+        c1 = e >= 8u ? z3 : z1;
+        c0 = e >= 16u ? z4 : c0;
+        c1 = e >= 16u ? z5 : c1;
+        at += e >> 3;
+        m = e & 7u;
     }
     // Append a token of up to 8 bytes (zero past its length).
     __device__ __forceinline__ void put8(const uint2 t, u32 len) {
         const u32 sh = m * 8u;
-        const u32 s0 = c | __funnelshift_l(0u, t.x, sh), s1 = __funnelshift_l(t.x, t.y, sh),
-                  s2 = __funnelshift_l(t.y, 0u, sh);
+        const bool q = (m & 4u) != 0u;
+        const u32 y0 = __funnelshift_l(0u, t.x, sh), y1 = __funnelshift_l(t.x, t.y, sh),
+                  y2 = __funnelshift_l(t.y, 0u, sh);
+        const u32 z0 = c0 | (q ? 0u : y0), z1 = c1 | (q ? y0 : y1), z2 = q ? y1 : y2, z3 = q ? y2 : 0u;
         const u32 e = m + len;
-        if (e >= 4u) at[0] = s0;
-        if (e >= 8u) at[1] = s1;
-        c = e >= 4u ? s1 : s0;
-        c = e >= 8u ? s2 : c;
-        at += e >> 2;
-        m = e & 3u;
+        if (e >= 8u) *reinterpret_cast<uint2*>(at) = make_uint2(z0, z1);
+        c0 = e >= 8u ? z2 : z0;
+        c1 = e >= 8u ? z3 : z1;
+        at += e >> 3;
+        m = e & 7u;
     }
     // The lane's bytes of a word that a following lane completed (every lane
     // of the warp has stored its words).
     __device__ __forceinline__ void finish() {
-        if (c) atomicOr(at, c);
+        u32* a = reinterpret_cast<u32*>(at);
+        if (c0) atomicOr(a, c0);
+        if (c1) atomicOr(a + 1, c1);
     }
 };
 
@@ -855,7 +861,7 @@ struct WarpCore {
                 else assemble<false>(p, dict, r, cw, lit, w0, w1);
             }
             // the round's last word is completed by no lane: its bytes are only added
-            if (lane == 0u && (nb & 3u)) stage[nb >> 2] = 0u;
+            if (lane == 0u && (nb & 7u)) reinterpret_cast<u64*>(stage)[nb >> 3] = 0ull;
             __syncwarp();
             if (in) {
                 w0.finish();
