@@ -67,7 +67,7 @@ SERVE_WORKLOADS = {
 }
 METRIC = "decoded GB/s (single-column decode, inputs resident in HBM)"
 SERVE_METRIC = "served decode: aggregate decoded GB/s at the offered load, with p50/p99 latency"
-SERVE_DEFAULT_CONFIG = 4   # the library's default batch configuration (warp tiles, one block of 16 warps per SM)
+SERVE_DEFAULT_CONFIG = 5   # the library's default batch configuration (staged units)
 BATCH_METRIC = "decoded GB/s (batched decode of many chunks, inputs resident in HBM)"
 L2_BYTES = 126 * 1024 * 1024
 
@@ -152,6 +152,13 @@ def load_traffic(workload: str):
     except Exception:
         return None
     return None
+
+
+def batch_launches(config: dict, codecs: int) -> int:
+    """Kernel launches of one batched decode in a configuration."""
+    if config["staged"]:
+        return 2 * codecs + 2
+    return 4 if config["warp_tiles"] else 2
 
 
 class ClockSampler:
@@ -720,7 +727,7 @@ def run_rows(args, rank, world, local_rank):
                      "frac": round(alg / avg_s / 1e9 / peak, 4), "peak_kind": peak_kind, "traffic": None,
                      "algorithmic_bytes_per_launch": int(alg), "kernel_ms": round(avg_s * 1e3, 4)},
         "clocks": clocks,
-        "gpu_launches": 7 * args.steps,   # row sums, their scan, row offsets, gather; reduce, tile scan, decode
+        "gpu_launches": 6 * args.steps,   # row sums, row offsets, gather; reduce, tile scan, decode
     }
     line.update(extra)
     print(json.dumps(line), flush=True)
@@ -986,8 +993,10 @@ def run_batched(args, rank, world, local_rank):
                      "traffic": load_traffic(args.workload), "algorithmic_bytes_per_launch": alg,
                      "kernel_ms": round(avg_s * 1e3, 4)},
         "clocks": clocks,
-        # per step one graph: index pass [+ reduce + tile scan] + the persistent decode kernel
-        "gpu_launches": (4 if fp.batch_config_info(pinfo["config"])["warp_tiles"] else 2) * args.steps,
+        # per step one graph: index pass [+ reduce + tile scan] + the persistent decode kernel; staged: a
+        # reduce and a decode per codec
+        "gpu_launches": batch_launches(fp.batch_config_info(pinfo["config"]), len({c.codec for c in plan._keep[1]}))
+                        * args.steps,
     }
     line.update(extra)
     if "e2e" not in line:
@@ -1373,8 +1382,9 @@ def run_served(args, rank, world, local_rank):
                    "generation_s": round(t_gen, 1), "parallelism": "single GPU",
                    "ms_per_step": "mean request latency"},
         "clocks": clocks,
-        # per wave: index pass [+ reduce + tile scan] + the persistent decode kernel
-        "gpu_launches": (4 if fp.batch_config_info(serve_cfg)["warp_tiles"] else 2) * waves,
+        # per wave: index pass [+ reduce + tile scan] + the persistent decode kernel; staged: a reduce and a
+        # decode per codec in the wave, counted here for waves of one codec (two more for each further one)
+        "gpu_launches": batch_launches(fp.batch_config_info(serve_cfg), 1) * waves,
     }
     line.update(extra)
     if "e2e" not in line:

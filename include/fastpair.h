@@ -415,9 +415,10 @@ fp_status fp_plan_destroy(fp_plan* plan);
 
 /* Batch configurations: slots per thread per codec (OnPair-16, OnPair-12,
  * FSST-8), blocks per SM, and 1 for the warp-tile decoder (index pass,
- * reduce, tile scan and a persistent decode: four launches) or 0 for the
- * block pipeline (index pass and the persistent decode).  Out pointers may be
- * NULL.  FSST-12 chunks are decoded only by the warp-tile configurations
+ * reduce, tile scan and a persistent decode: four launches), 2 for its staged
+ * form (a reduce per codec, index pass, tile scan, a decode per codec; tables
+ * in shared memory) or 0 for the block pipeline (index pass and the
+ * persistent decode).  Out pointers may be NULL.  FSST-12 chunks are decoded only by the warp-tile configurations
  * (with the OnPair-12 slots per thread); fp_plan_create skips the others for
  * plans that hold FSST-12 chunks and fp_plan_create_config rejects them with
  * FP_ERR_ARG. */

@@ -542,7 +542,8 @@ def batch_config_info(config: int) -> dict:
     b, w = ctypes.c_uint32(), ctypes.c_uint32()
     _check(lib().fp_batch_config_info(config, ctypes.cast(k, ctypes.c_void_p), ctypes.byref(b), ctypes.byref(w)),
            "fp_batch_config_info")
-    return {"slots_per_thread": list(k), "blocks_per_sm": b.value, "warp_tiles": bool(w.value)}
+    return {"slots_per_thread": list(k), "blocks_per_sm": b.value, "warp_tiles": bool(w.value),
+            "staged": w.value == 2}
 
 
 # ---- served decode (fp_serve_*) ----------------------------------------------

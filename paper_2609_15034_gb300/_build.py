@@ -38,7 +38,7 @@ def nvcc() -> str:
 # traffic counters taken on one build stay valid while these and the build
 # flags are unchanged.
 DECODE_PATH = ["fp_api.cu", "fp_decode.cu", "fp_var16.cu", "fp_var12.cu", "fp_var8.cu", "fp_var12f.cu", "fp_varpk.cu",
-               "fp_variants.cuh", "fp_decoder.cuh", "fp_internal.h", "fp_warp.cuh"]
+               "fp_variants.cuh", "fp_decoder.cuh", "fp_internal.h", "fp_warp.cuh", "fp_reduce.cuh", "fp_cluster.cuh"]
 
 
 def decode_path_digest() -> str:

@@ -13,8 +13,9 @@
 // index, data-error word and decoded size.  The decode block copies the
 // chunk's record (SlotSrc) into its ring slot with the tile's inputs, so
 // consecutive tiles of one block may belong to different chunks and codecs.
-// Dictionaries are read through the L1 cache (a per-chunk copy into shared
-// memory would have to be repeated at every chunk change).
+// Dictionaries are read through the L1 cache here (a copy into shared memory
+// would have to be repeated at every chunk change); the staged configuration
+// below cuts the chunks into units so that it pays.
 //
 // Autotuning.  The tile shape (code slots per thread for each codec) and
 // the blocks per SM are compiled or launch-time choices; fp_plan_create
@@ -29,6 +30,7 @@
 #include <string>
 #include <vector>
 
+#include "fp_reduce.cuh"
 #include "fp_warp.cuh"
 
 namespace fp {
@@ -63,8 +65,10 @@ __global__ void __launch_bounds__(256) batch_index_kernel(const IdxParams ip) {
         cs->x.c_end = x.c_end;
         cs->x.bad = x.bad;
     }
-    index_groups(p, x, (u32)(__ffs((int)ip.tile[q]) - 1), b.start, (u64)b.start + kIdxPerBlock, threadIdx.x, 256,
-                 const_cast<u32*>(p.first));
+    static_assert(kIdxPerBlock == 8 * 256, "a chunk of 256 boundaries per warp");
+    index_by_warps(p, x, (u32)(__ffs((int)ip.tile[q]) - 1), b.start / 256u + (threadIdx.x >> 5), 0x7fffffffu,
+                   const_cast<u32*>(p.first));
+    grid_wait();   // staged batches start this beside the reduce
 }
 
 template <int K16, int K12, int K8, int MINB>
@@ -254,6 +258,194 @@ __global__ void __launch_bounds__(NW * 32, MINB) wbatch_decode_kernel(const Batc
     decode_queue<FP_FSST12, K12>(bp, 3, gw, bp.q[3].n_tiles, W, mine, rs, bar, phase);
 }
 
+// ---------------------------------------------------------------------------
+// Staged batches: index pass, reduce and tile scan as above, then one decode
+// launch per codec in which a block takes units -- runs of up to kUnitTiles
+// tiles of one chunk, by ticket, the largest first -- and stages the chunk's
+// tables in shared memory as the single-column decode does.  Against reading
+// them through L1 (wbatch_decode_kernel): what bounds that one is the L1 data
+// pipe, where a gather of 32 lengths or tokens costs 10 to 20 wavefronts
+// instead of 3 to 10.  Staging a unit's tables (4 to 68 KiB) takes a block
+// about 2 us, its 128 tiles about 40.  Units of 64 or 256 tiles: 543 and 537
+// us on the 256-chunk batch against 527 (with the reduce still through L1).
+// ---------------------------------------------------------------------------
+constexpr u64 kUnitTiles = 128;
+constexpr int kUnitWarps = 16;
+
+template <int CODEC, int K>
+struct UnitShape {
+    static constexpr bool DSMEM = CODEC != FP_ONPAIR16;
+    typedef WarpCore<CODEC, K, DSMEM, (CODEC == FP_ONPAIR16 || CODEC == FP_ONPAIR12) ? 16 : 8, false, true> C;
+    static constexpr size_t SMEM = (size_t)C::STAGED_BYTES + kUnitWarps * sizeof(typename C::Area);
+};
+
+template <int CODEC, int K>
+__global__ void __launch_bounds__(kUnitWarps * 32, 1) unit_decode_kernel(const BatchParams bp) {
+    typedef UnitShape<CODEC, K> S;
+    typedef typename S::C C;
+    constexpr int q = CODEC - 1;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) u64 s_bar;
+    __shared__ __align__(8) u64 s_code_bar[kUnitWarps];
+    __shared__ SlotSrc rec;
+    __shared__ uint4 s_unit[2];   // this unit, the next one
+    uint4* s_dict = reinterpret_cast<uint4*>(smem_raw);
+    uint8_t* s_lens = smem_raw + C::DICT_BYTES;
+    const u32 lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    typename C::Area& area = reinterpret_cast<typename C::Area*>(smem_raw + C::STAGED_BYTES)[warp];
+    typename C::CodeBar cb;
+    cb.init(s_code_bar + warp);
+    // the codecs' launches overlap (they share nothing but finished tables);
+    // each ends only after the one before it
+    grid_release();
+    const u32 n_units = bp.n_units[q];
+    auto take = [&]() -> uint4 {
+        const u32 u = atomicAdd(&bp.ws->unit_counter[q], 1u);
+        return u < n_units ? __ldg(bp.units[q] + u) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    if (threadIdx.x == 0) {
+        mbar_init(&s_bar, 1u);
+        mbar_init_fence();
+        s_unit[0] = take();
+    }
+    __syncthreads();
+    const void* staged = nullptr;   // the table in shared memory
+    u32 bar_phase = 0u;
+    for (u32 i = 0;; ++i) {
+        const uint4 unit = s_unit[i & 1u];
+        if (unit.z == 0u) break;
+        const SlotSrc* src = bp.q[q].src + unit.x;
+        if (threadIdx.x < sizeof(SlotSrc) / 16) reinterpret_cast<uint4*>(&rec)[threadIdx.x] = reinterpret_cast<const uint4*>(src)[threadIdx.x];
+        if (threadIdx.x == 32) s_unit[(i & 1u) ^ 1u] = take();   // in flight during the unit
+        __syncthreads();
+        const DecodeParams& p = rec.p;
+        if (p.dict.table != staged) {
+            const bool aligned =
+                ((reinterpret_cast<uintptr_t>(p.dict.table) | reinterpret_cast<uintptr_t>(p.dict.lens)) & 15u) == 0u;
+            if (C::BULK_STAGE && aligned) {
+                if (threadIdx.x == 0) C::bulk_tables(p, s_dict, s_lens, &s_bar);
+                mbar_wait(&s_bar, bar_phase, p.ws);
+                bar_phase ^= 1u;
+            } else {
+                C::stage_dict(p, s_dict, s_lens, kUnitWarps * 32);
+                __syncthreads();
+            }
+            staged = p.dict.table;
+        }
+        const u64* ex = bp.ex + rec.wt_base;
+        u32 err = 0;
+        u64 t = unit.y + warp;
+        const u64 t_end = (u64)unit.y + unit.z;
+        if (t < t_end) {
+            typename C::Fetch cur;
+            C::fetch(p, rec.x, ex, t, area, cb, cur);
+            for (; t < t_end; t += kUnitWarps) {
+                typename C::Fetch nxt;
+                C::decode_tile(p, rec.x, t, cur, ex, s_dict, s_lens, area, cb, err, [&] {
+                    if (t + kUnitWarps < t_end) C::fetch(p, rec.x, ex, t + kUnitWarps, area, cb, nxt);
+                });
+                cur = nxt;
+            }
+            if (err) atomicOr(p.err_word, err);
+        }
+        __syncthreads();   // the tables and the record are replaced
+    }
+    C::stage_free(lane);
+    grid_wait();
+}
+
+// Reduce of a staged batch: units as in the decode, two blocks per SM, the
+// lengths in shared memory (OnPair-16 and FSST-8 in the tables of
+// fp_reduce.cuh).  Extents come from the offsets themselves, so the index pass
+// runs beside it (256 chunks: 527 -> 471 us per call).
+template <int CODEC, int K>
+struct UnitReduce {
+    static constexpr bool TABLE = CODEC == FP_ONPAIR16 || CODEC == FP_FSST8;
+    typedef WarpCore<CODEC, K, !TABLE, (CODEC == FP_ONPAIR16 || CODEC == FP_ONPAIR12) ? 16 : 8, false, true> C;
+    static constexpr size_t SMEM = TABLE ? 65536 : C::LENS_BYTES;
+};
+
+template <int CODEC, int K>
+__global__ void __launch_bounds__(512, 2) unit_reduce_kernel(const BatchParams bp) {
+    typedef UnitReduce<CODEC, K> U;
+    typedef typename U::C C;
+    constexpr int q = CODEC - 1;
+    extern __shared__ __align__(128) unsigned char tab[];
+    __shared__ SlotSrc rec;
+    __shared__ uint4 s_unit[2];
+    const u32 lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    grid_release();
+    const u32 n_units = bp.n_units[q];
+    auto take = [&]() -> uint4 {
+        const u32 u = atomicAdd(&bp.ws->reduce_counter[q], 1u);
+        return u < n_units ? __ldg(bp.units[q] + u) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    if (threadIdx.x == 0) s_unit[0] = take();
+    __syncthreads();
+    const void* staged = nullptr;
+    for (u32 i = 0;; ++i) {
+        const uint4 unit = s_unit[i & 1u];
+        if (unit.z == 0u) break;
+        const SlotSrc* src = bp.q[q].src + unit.x;
+        if (threadIdx.x < sizeof(SlotSrc) / 16) reinterpret_cast<uint4*>(&rec)[threadIdx.x] = reinterpret_cast<const uint4*>(src)[threadIdx.x];
+        if (threadIdx.x == 32) s_unit[(i & 1u) ^ 1u] = take();
+        __syncthreads();
+        const DecodeParams& p = rec.p;
+        if (p.dict.lens != staged) {
+            if constexpr (U::TABLE) {
+                LengthTable<CODEC, K>::fill(p, tab);
+            } else {
+                const u32* lsrc = reinterpret_cast<const u32*>(p.dict.lens);
+                for (u32 k = threadIdx.x; k < C::LENS_BYTES / 4; k += blockDim.x) reinterpret_cast<u32*>(tab)[k] = __ldg(lsrc + k);
+            }
+            staged = p.dict.lens;
+            __syncthreads();
+        }
+        Extent x;
+        x.first_tile = 0;
+        x.n_tiles = rec.x.n_tiles;
+        slot_range(p, x);
+        // tiles [t_lo, t_hi) lie wholly inside the column (and so inside the buffer)
+        const u32 t_lo = (u32)((x.c_begin + C::TILE - 1) / C::TILE), t_hi = (u32)(x.c_end / C::TILE);
+        u64* const agg = bp.agg + rec.wt_base;
+        u32 err = 0;
+        const u32 t_end = unit.y + unit.z;
+        u32 t = unit.y + warp;
+        u32 nv[C::LANE_WORDS];
+        bool nin = t < t_end && C::load_fast(p, C::lane_q0(x, t), nv);
+        for (; t < t_end; t += 16u) {
+            u32 wv[1][C::LANE_WORDS];
+#pragma unroll
+            for (int k = 0; k < C::LANE_WORDS; ++k) wv[0][k] = nv[k];
+            const bool in = nin;
+            nin = t + 16u < t_end && C::load_fast(p, C::lane_q0(x, t + 16u), nv);
+            u64 e;
+            if (t >= t_lo && t < t_hi) {
+                if constexpr (CODEC == FP_FSST8) {
+                    u64 r[1];
+                    LengthTable<CODEC, K>::template elements<1>(wv, tab, lane, err, r);
+                    e = r[0];
+                } else {
+                    u32 sum;
+                    if constexpr (U::TABLE) sum = LengthTable<CODEC, K>::lane_sum(wv[0], tab, lane * 4u, err);
+                    else sum = C::lane_length_sum(wv[0], tab, err);
+                    sum = __reduce_add_sync(0xffffffffu, sum);
+                    e = wt_pack<true>(TElem{sum, sum, 2u});
+                }
+            } else {
+                typedef WarpCore<CODEC, K, false> E;   // lengths through L1
+                typename E::R r;
+                E::finish_load(p, x, E::lane_q0(x, t), wv[0], in, p.dict.lens, r);
+                e = wt_pack<true>(E::tile_element(r, lane, err));
+            }
+            if (lane == 31) agg[t] = e;
+        }
+        if (err) atomicOr(p.err_word, err);
+        __syncthreads();   // the table and the record are replaced
+    }
+    grid_wait();
+}
+
 template <int K16, int K12, int K8, int NW>
 constexpr size_t wbatch_smem() {
     return (size_t)NW * ((WarpSlot<K16, K12, K8>::bytes + sizeof(SlotSrc) + 15) / 16 * 16);
@@ -268,6 +460,11 @@ struct BatchKernel {
     int threads;         // threads per block of the decode kernel
     const void* reduce;
     const void* scan;
+    // staged: a decode kernel per queue (`kernel` is the first of them), tables in shared memory
+    const void* unit[kQueues];
+    size_t unit_smem[kQueues];
+    const void* unit_reduce[kQueues];
+    size_t unit_reduce_smem[kQueues];
 };
 
 template <int K16, int K12, int K8, int MINB>
@@ -299,12 +496,37 @@ BatchKernel make_wbatch_kernel() {
     return k;
 }
 
+template <int K16, int K12, int K8>
+BatchKernel make_unit_kernels() {
+    BatchKernel k = make_wbatch_kernel<K16, K12, K8, kUnitWarps, 1>();
+    k.unit[0] = (const void*)&unit_decode_kernel<FP_ONPAIR16, K16>;
+    k.unit[1] = (const void*)&unit_decode_kernel<FP_ONPAIR12, K12>;
+    k.unit[2] = (const void*)&unit_decode_kernel<FP_FSST8, K8>;
+    k.unit[3] = (const void*)&unit_decode_kernel<FP_FSST12, K12>;
+    k.unit_smem[0] = UnitShape<FP_ONPAIR16, K16>::SMEM;
+    k.unit_smem[1] = UnitShape<FP_ONPAIR12, K12>::SMEM;
+    k.unit_smem[2] = UnitShape<FP_FSST8, K8>::SMEM;
+    k.unit_smem[3] = UnitShape<FP_FSST12, K12>::SMEM;
+    k.unit_reduce[0] = (const void*)&unit_reduce_kernel<FP_ONPAIR16, K16>;
+    k.unit_reduce[1] = (const void*)&unit_reduce_kernel<FP_ONPAIR12, K12>;
+    k.unit_reduce[2] = (const void*)&unit_reduce_kernel<FP_FSST8, K8>;
+    k.unit_reduce[3] = (const void*)&unit_reduce_kernel<FP_FSST12, K12>;
+    k.unit_reduce_smem[0] = UnitReduce<FP_ONPAIR16, K16>::SMEM;
+    k.unit_reduce_smem[1] = UnitReduce<FP_ONPAIR12, K12>::SMEM;
+    k.unit_reduce_smem[2] = UnitReduce<FP_FSST8, K8>::SMEM;
+    k.unit_reduce_smem[3] = UnitReduce<FP_FSST12, K12>::SMEM;
+    k.kernel = k.unit[0];
+    k.smem_bytes = k.unit_smem[0];
+    return k;
+}
+
 const std::vector<BatchKernel>& batch_kernels() {
     static const std::vector<BatchKernel> v = {
         make_batch_kernel<16, 16, 16, 2>(),
         make_batch_kernel<8, 8, 16, 2>(),
         make_wbatch_kernel<16, 16, 32, 8, 2>(),
         make_wbatch_kernel<16, 16, 32, 16, 1>(),
+        make_unit_kernels<16, 16, 32>(),
     };
     return v;
 }
@@ -315,7 +537,7 @@ struct Config {
     int bps;      // blocks per SM launched (<= what fits)
 };
 const std::vector<Config>& configs() {
-    static const std::vector<Config> v = {{0, 2}, {0, 1}, {1, 2}, {2, 2}, {3, 1}};
+    static const std::vector<Config> v = {{0, 2}, {0, 1}, {1, 2}, {2, 2}, {3, 1}, {4, 1}};
     return v;
 }
 
@@ -362,12 +584,12 @@ namespace {
 // writes the fourth and the look-back words are tagged per launch.
 struct LayoutImage {
     std::vector<char> bytes;
-    size_t o_src[kQueues], o_tc[kQueues], o_ib, o_sb, o_first, o_ts, o_agg, o_ex, table_bytes, total_bytes;
+    size_t o_src[kQueues], o_tc[kQueues], o_un[kQueues], o_ib, o_sb, o_first, o_ts, o_agg, o_ex, table_bytes, total_bytes;
     uint64_t total_tiles = 0;
     uint64_t status_words = 0;   // look-back words (per tile, or per tile-scan block with warp tiles)
     uint32_t n_idx = 0;
     uint32_t n_sb = 0;           // tile-scan blocks (warp tiles)
-    uint32_t n_tiles_q[kQueues], n_chunks_q[kQueues];
+    uint32_t n_tiles_q[kQueues], n_chunks_q[kQueues], n_units_q[kQueues];
     uint64_t slots_q[kQueues];
 };
 
@@ -377,7 +599,7 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // d_status[i] / d_total[i].  Device addresses inside the records are
 // offsets until relocate() adds the layout's base.
 fp_status make_layout(const fp_chunk* chunks, uint32_t n, const BatchKernel& BK, uint32_t* d_status,
-                      unsigned long long* d_total, WsHeader* ws, LayoutImage& L) {
+                      unsigned long long* d_total, WsHeader* ws, int sms, LayoutImage& L) {
     std::vector<uint32_t> qlist[kQueues];
     for (uint32_t i = 0; i < n; ++i) qlist[chunks[i].codec - 1].push_back(i);
     if (!qlist[3].empty() && BK.k[3] == 0)
@@ -386,7 +608,14 @@ fp_status make_layout(const fp_chunk* chunks, uint32_t n, const BatchKernel& BK,
     std::vector<uint32_t> tchunk[kQueues];
     std::vector<IdxBlock> iblk;
     std::vector<uint2> sblk;
+    std::vector<uint4> units[kQueues];
     uint64_t tile_glob = 0, first_glob = 0, sb_glob = 0;
+    // tiles of a unit: about eight units per SM and a tile for every warp, at most kUnitTiles
+    uint64_t unit_tiles = 0;
+    for (uint32_t i = 0; i < n; ++i)
+        unit_tiles += max_slots_of(chunks[i].codec, chunks[i].codes_bytes) / (32u * std::max(BK.k[chunks[i].codec - 1], 8));
+    unit_tiles = unit_tiles / ((uint64_t)sms * 8) / kUnitWarps * kUnitWarps;
+    unit_tiles = std::min<uint64_t>(std::max<uint64_t>(unit_tiles, kUnitWarps), kUnitTiles);
     for (int q = 0; q < kQueues; ++q) {
         const int codec = q + 1;
         const uint64_t T = (uint64_t)(BK.warp_tiles ? 32 : kWork) * (uint64_t)BK.k[q];
@@ -430,6 +659,13 @@ fp_status make_layout(const fp_chunk* chunks, uint32_t n, const BatchKernel& BK,
             sb_glob += n_sb;
             src[q].push_back(s);
             tchunk[q].insert(tchunk[q].end(), nt, ci);
+            if (BK.unit[q]) {
+                const uint64_t nu = (nt + unit_tiles - 1) / unit_tiles;   // equal parts
+                for (uint64_t u = 0; u < nu; ++u) {
+                    const uint64_t t0 = nt * u / nu, t1 = nt * (u + 1) / nu;
+                    units[q].push_back(make_uint4(ci, (uint32_t)t0, (uint32_t)(t1 - t0), 0u));
+                }
+            }
             const uint64_t nb = (uint64_t)c.n_strings + 1;
             for (uint64_t st = 0; st < nb; st += kIdxPerBlock)
                 iblk.push_back(IdxBlock{((uint32_t)q << 30) | ci, (uint32_t)st});
@@ -439,11 +675,15 @@ fp_status make_layout(const fp_chunk* chunks, uint32_t n, const BatchKernel& BK,
         }
         L.n_tiles_q[q] = tile_q;
         L.n_chunks_q[q] = (uint32_t)src[q].size();
+        // largest first; a chunk's units stay together, so that a block often finds its table staged
+        std::stable_sort(units[q].begin(), units[q].end(), [](const uint4& a, const uint4& b) { return a.z / 16 > b.z / 16; });
+        L.n_units_q[q] = (uint32_t)units[q].size();
     }
     if (iblk.size() > 0x7fffffffull) return fail(FP_ERR_ARG, "batch has too many strings");
     size_t off = 0;
     for (int q = 0; q < kQueues; ++q) { L.o_src[q] = off; off = align256(off + src[q].size() * sizeof(SlotSrc)); }
     for (int q = 0; q < kQueues; ++q) { L.o_tc[q] = off; off = align256(off + tchunk[q].size() * sizeof(uint32_t)); }
+    for (int q = 0; q < kQueues; ++q) { L.o_un[q] = off; off = align256(off + units[q].size() * sizeof(uint4)); }
     L.o_ib = off; off = align256(off + iblk.size() * sizeof(IdxBlock));
     L.o_sb = off; off = align256(off + sblk.size() * sizeof(uint2));
     L.table_bytes = off;
@@ -459,6 +699,7 @@ fp_status make_layout(const fp_chunk* chunks, uint32_t n, const BatchKernel& BK,
     L.bytes.assign(L.table_bytes, 0);
     for (int q = 0; q < kQueues; ++q) {
         if (!src[q].empty()) memcpy(&L.bytes[L.o_src[q]], src[q].data(), src[q].size() * sizeof(SlotSrc));
+        if (!units[q].empty()) memcpy(&L.bytes[L.o_un[q]], units[q].data(), units[q].size() * sizeof(uint4));
         if (!tchunk[q].empty()) memcpy(&L.bytes[L.o_tc[q]], tchunk[q].data(), tchunk[q].size() * sizeof(uint32_t));
     }
     if (!iblk.empty()) memcpy(&L.bytes[L.o_ib], iblk.data(), iblk.size() * sizeof(IdxBlock));
@@ -482,6 +723,13 @@ void relocate(LayoutImage& L, char* base) {
 fp_status launch_shape(const LayoutImage& L, const BatchKernel& BK, int bps_limit, int sms, int* grid_out,
                        uint32_t split[2]) {
     cudaError_t e = cudaFuncSetAttribute(BK.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BK.smem_bytes);
+    for (int q = 0; q < kQueues && e == cudaSuccess; ++q)
+        if (BK.unit[q]) {
+            e = cudaFuncSetAttribute(BK.unit[q], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BK.unit_smem[q]);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(BK.unit_reduce[q], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)BK.unit_reduce_smem[q]);
+        }
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(batch)");
     int fit = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, BK.kernel, BK.threads, BK.smem_bytes);
@@ -519,6 +767,8 @@ void make_params(const LayoutImage& L, const BatchKernel& BK, char* base, WsHead
         bp.q[q].tile_chunk = reinterpret_cast<const uint32_t*>(base + L.o_tc[q]);
         bp.q[q].n_tiles = L.n_tiles_q[q];
         bp.q[q].n_chunks = L.n_chunks_q[q];
+        bp.units[q] = reinterpret_cast<const uint4*>(base + L.o_un[q]);
+        bp.n_units[q] = L.n_units_q[q];
     }
     bp.split[0] = split[0];
     bp.split[1] = split[1];
@@ -536,21 +786,63 @@ void make_params(const LayoutImage& L, const BatchKernel& BK, char* base, WsHead
     }
 }
 
+cudaError_t launch_scan(const BatchKernel& BK, const BatchParams& bp, int sms, void** args, cudaStream_t stream) {
+    uint32_t sg = bp.n_scan_blocks < (uint32_t)(sms * 2) ? bp.n_scan_blocks : (uint32_t)(sms * 2);
+    if (sg < 1) sg = 1;
+    return cudaLaunchKernel(BK.scan, dim3(sg), dim3(256), args, 0, stream);
+}
+
 cudaError_t launch_kernels(const BatchKernel& BK, const BatchParams& bp, const IdxParams& ip, uint32_t n_idx, int grid,
                            int sms, cudaStream_t stream) {
     void* iargs[] = {(void*)&ip};
-    cudaError_t e = cudaLaunchKernel((const void*)&batch_index_kernel, dim3(n_idx), dim3(256), iargs, 0, stream);
-    if (e != cudaSuccess) return e;
     void* args[] = {(void*)&bp};
-    if (BK.warp_tiles) {
-        e = cudaLaunchKernel(BK.reduce, dim3((unsigned)(sms * 3)), dim3(256), args, 0, stream);
+    cudaError_t e;
+    if (!BK.unit[0]) {
+        e = cudaLaunchKernel((const void*)&batch_index_kernel, dim3(n_idx), dim3(256), iargs, 0, stream);
         if (e != cudaSuccess) return e;
-        uint32_t sg = bp.n_scan_blocks < (uint32_t)(sms * 2) ? bp.n_scan_blocks : (uint32_t)(sms * 2);
-        if (sg < 1) sg = 1;
-        e = cudaLaunchKernel(BK.scan, dim3(sg), dim3(256), args, 0, stream);
-        if (e != cudaSuccess) return e;
+        if (BK.warp_tiles) {
+            e = cudaLaunchKernel(BK.reduce, dim3((unsigned)(sms * 3)), dim3(256), args, 0, stream);
+            if (e != cudaSuccess) return e;
+            e = launch_scan(BK, bp, sms, args, stream);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaLaunchKernel(BK.kernel, dim3(grid), dim3(BK.threads), args, BK.smem_bytes, stream);
     }
-    return cudaLaunchKernel(BK.kernel, dim3(grid), dim3(BK.threads), args, BK.smem_bytes, stream);
+    // Staged: a reduce per codec and the index pass, the scan, a decode per
+    // codec.  Inside each of the two groups a launch may start in the tail of
+    // the one before it (they share nothing; each ends only after that one).
+    auto launch = [&](const void* k, uint32_t blocks, int threads, size_t smem, void** a, bool early) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(blocks);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = early ? 1 : 0;
+        return cudaLaunchKernelExC(&cfg, k, a);
+    };
+    bool early = false;
+    for (int q = 0; q < kQueues; ++q) {
+        if (!bp.n_units[q]) continue;
+        e = launch(BK.unit_reduce[q], std::min(bp.n_units[q], (uint32_t)sms * 2), 512, BK.unit_reduce_smem[q], args, early);
+        if (e != cudaSuccess) return e;
+        early = true;
+    }
+    e = launch((const void*)&batch_index_kernel, n_idx, 256, 0, iargs, true);
+    if (e != cudaSuccess) return e;
+    e = launch_scan(BK, bp, sms, args, stream);
+    if (e != cudaSuccess) return e;
+    early = false;
+    for (int q = 0; q < kQueues; ++q) {
+        if (!bp.n_units[q]) continue;
+        e = launch(BK.unit[q], std::min(bp.n_units[q], (uint32_t)grid), kUnitWarps * 32, BK.unit_smem[q], args, early);
+        if (e != cudaSuccess) return e;
+        early = true;
+    }
+    return cudaSuccess;
 }
 
 // Lay out configuration `cfg` for a plan (fresh device memory, zeroed
@@ -560,7 +852,7 @@ fp_status build_layout(fp_plan* P, int cfg) {
     const BatchKernel& BK = batch_kernels()[C.kernel];
     LayoutImage L;
     fp_status st = make_layout(P->chunks.data(), (uint32_t)P->chunks.size(), BK, P->d_status, P->d_total,
-                               static_cast<WsHeader*>(P->d_hdr), L);
+                               static_cast<WsHeader*>(P->d_hdr), P->sms, L);
     if (st != FP_OK) return st;
     if (P->d_layout) {
         cudaFree(P->d_layout);
@@ -615,7 +907,7 @@ std::string plan_signature(const fp_plan* P) {
     mix((uint32_t)P->sms);
     for (uint32_t k : keys) mix(k);
     char buf[64];
-    snprintf(buf, sizeof(buf), "b1-%016llx-%zu", (unsigned long long)h, P->chunks.size());
+    snprintf(buf, sizeof(buf), "b2-%016llx-%zu", (unsigned long long)h, P->chunks.size());
     return buf;
 }
 
@@ -773,10 +1065,10 @@ fp_status plan_create(const fp_chunk* chunks, uint32_t n, int force_cfg, const c
 
 namespace fp {
 
-// Warp tiles (16/16/32 slots per lane, one block of 16 warps per SM): the
-// fastest configuration on the mixed 4,096-chunk batch (41 ms, against 50 ms
-// for two blocks of 8 warps and 55 ms for the block pipeline).
-int batch_config_default() { return 4; }
+// Staged units: the fastest configuration on every mixed batch measured (256
+// chunks of 4 KB - 16 MB: 471 us against 602 us for warp tiles through L1; 60
+// chunks up to 1 MB: 48 against 55; 16 up to 4 MB: 37 against 57).
+int batch_config_default() { return 5; }
 
 fp_status wave_init(WaveBuffers& W, uint32_t cap_chunks) {
     int dev = 0;
@@ -821,7 +1113,7 @@ fp_status wave_launch(WaveBuffers& W, const fp_chunk* chunks, uint32_t n, int co
     const BatchKernel& BK = batch_kernels()[C.kernel];
     LayoutImage L;
     WsHeader* ws = static_cast<WsHeader*>(W.d_hdr);
-    fp_status st = make_layout(chunks, n, BK, W.d_status, W.d_total, ws, L);
+    fp_status st = make_layout(chunks, n, BK, W.d_status, W.d_total, ws, W.sms, L);
     if (st != FP_OK) return st;
     cudaError_t e;
     if (L.total_bytes > W.layout_cap) {
@@ -983,7 +1275,7 @@ fp_status fp_batch_config_info(int config, uint32_t* slots_per_thread3, uint32_t
     if (slots_per_thread3)
         for (int q = 0; q < 3; ++q) slots_per_thread3[q] = (uint32_t)BK.k[q];
     if (blocks_per_sm) *blocks_per_sm = (uint32_t)C.bps;
-    if (warp_tiles) *warp_tiles = (uint32_t)BK.warp_tiles;
+    if (warp_tiles) *warp_tiles = BK.unit[0] ? 2u : (uint32_t)BK.warp_tiles;
     return FP_OK;
 }
 

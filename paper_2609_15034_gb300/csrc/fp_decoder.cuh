@@ -780,6 +780,7 @@ __device__ __forceinline__ void finish_launch(WsHeader* ws, u32 epoch) {
             ws->queue_counter[0] = 0;
             ws->queue_counter[1] = 0;
             ws->queue_counter[2] = 0;
+            for (int q = 0; q < 4; ++q) ws->unit_counter[q] = ws->reduce_counter[q] = 0;
             ws->exit_counter = 0;
             ws->abort = 0;
             ws->spin_limit = 0;

@@ -35,7 +35,9 @@ struct WsHeader {
     unsigned int spin_limit;     // polls before a look-back gives up (0 = the built-in limit); reset per launch
     unsigned int bar_count;      // one-launch decode: blocks arrived at the current grid barrier
     unsigned int bar_gen;        // one-launch decode: grid barriers passed
-    unsigned int pad[17];
+    unsigned int unit_counter[4];    // staged batch: next unit of each codec, decode
+    unsigned int reduce_counter[4];  // and reduce
+    unsigned int pad[9];
 };
 constexpr size_t kWsHeaderBytes = 128;
 static_assert(sizeof(WsHeader) == kWsHeaderBytes, "workspace header size");
@@ -123,6 +125,9 @@ struct BatchParams {
     const uint2* scan_blocks;       // (queue << 30 | chunk, block within the chunk) per tile-scan block
     uint32_t n_scan_blocks;
     uint32_t pad;
+    // staged batches only: (chunk of the queue, first tile, tiles, 0) per unit, the largest first
+    const uint4* units[kQueues];
+    uint32_t n_units[kQueues];
 };
 
 // A compiled decoder shape.

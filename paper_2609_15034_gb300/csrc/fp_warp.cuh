@@ -630,13 +630,17 @@ struct WarpCore {
         if (threadIdx.x == 0) {
             mbar_init(bar, 1u);
             mbar_init_fence();
-            mbar_expect_tx(bar, (u32)(DICT_BYTES + LENS_BYTES));
-            if (DSMEM) bulk_g2s(s_dict, p.dict.table, (u32)DICT_BYTES, bar);
-            bulk_g2s(s_lens, p.dict.lens, (u32)LENS_BYTES, bar);
-            mbar_arrive(bar);
+            bulk_tables(p, s_dict, s_lens, bar);
         }
         __syncthreads();   // the barrier is initialised before anyone waits on it
         mbar_wait(bar, 0u, p.ws);
+    }
+    // Issue the two copies (one thread; `bar` is initialised).
+    static __device__ __forceinline__ void bulk_tables(const DecodeParams& p, uint4* s_dict, uint8_t* s_lens, u64* bar) {
+        mbar_expect_tx(bar, (u32)(DICT_BYTES + LENS_BYTES));
+        if (DSMEM) bulk_g2s(s_dict, p.dict.table, (u32)DICT_BYTES, bar);
+        bulk_g2s(s_lens, p.dict.lens, (u32)LENS_BYTES, bar);
+        mbar_arrive(bar);
     }
 
     // Byte count of an escape-free lane whose K slots all lie inside the
