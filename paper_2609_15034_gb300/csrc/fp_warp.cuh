@@ -122,11 +122,11 @@ struct StageWriter {
 // decoded bytes, at the alignment they have in the output, so that the whole
 // 16-byte chunks leave by one bulk copy per tile (no store instructions, and
 // no scattered lines in L1).
-template <int K, int CAP, int CODE_BYTES, int SCRATCH>
+template <int K, int CAP, int CODE_BYTES>
 struct WarpArea {
     uint4 stage[CAP / 16 + 1];
     // code bytes of the tile to decode next (bulk copy), or the unpack's scratch (packed codes)
-    uint4 codes[CODE_BYTES + SCRATCH ? (CODE_BYTES + SCRATCH) / 16 : 1];
+    uint4 codes[CODE_BYTES ? CODE_BYTES / 16 : 1];
     u32 pre[K / 4][32];     // tile-relative output offset of slot 4m of each lane
     u32 contrib[K / 4][32]; // bytes each slot produced, one byte per slot
     u32 lit_mask[32];       // FSST-8: bit k = slot k holds a literal byte
@@ -152,13 +152,9 @@ struct WarpCore {
     static constexpr int TILE = 32 * K;
     static constexpr int WBITS = (CODEC == FP_ONPAIR16) ? 16 : (W12 ? 12 : 8);
     static constexpr int LANE_BYTES = K * WBITS / 8;   // code bytes of one lane
-    // words a lane loads: its code bytes, or for packed codes the 32-bit
-    // words covering K codes of up to 16 bits at any bit offset
-    static constexpr int LANE_WORDS = PACKED ? (K * 16 + 31) / 32 + 1 : LANE_BYTES / 4;
-    // per-lane scratch: word i next to word i + 1, as 8-byte pairs; a stride
-    // of 2 * LANE_WORDS words keeps the 16 lanes of each half-warp's 8-byte
-    // accesses on distinct banks
-    static constexpr int PK_STRIDE = 2 * LANE_WORDS;
+    // words a lane loads: its code bytes; for packed codes up to 16 codes of
+    // 16 bits, which begin at a word or in the middle of one (packed_words())
+    static constexpr int LANE_WORDS = PACKED ? K / 2 : LANE_BYTES / 4;
     // entries of the table (a staged table, or the global planes)
     static constexpr int kTable = (CODEC == FP_FSST8) ? 256 : (CODEC == FP_ONPAIR16 ? 65536 : 4096);
     // FSST-8 with a staged table: the symbols, then the 256 literal bytes as
@@ -177,7 +173,7 @@ struct WarpCore {
     // 576 us per call, FSST-12 documents 114 -> 105), 16-slot lanes are not
     // and only pay the wait (OnPair-12 10M 648 -> 659).
     static constexpr bool BULK_CODES = K == 32;
-    typedef WarpArea<K, CAP, BULK_CODES ? TILE_BYTES : 0, PACKED ? 32 * PK_STRIDE * 4 : 0> Area;
+    typedef WarpArea<K, CAP, BULK_CODES ? TILE_BYTES : 0> Area;
     static constexpr int LENS_BYTES = LSMEM ? kTable : 0;
     static constexpr int STAGED_BYTES = DICT_BYTES + LENS_BYTES;   // tables in front of the warp areas
     typedef TileRegs<CODEC, K> R;
@@ -213,10 +209,9 @@ struct WarpCore {
     static __device__ __forceinline__ bool load_fast(const DecodeParams& p, u64 q0, u32 (&wv)[LANE_WORDS]) {
         if (PACKED) {
             const u64 w0 = (q0 * p.packed_bits) >> 5;   // the word holding the lane's first bit
-            if ((w0 + LANE_WORDS) * 4 > p.codes_bytes) return false;
-            const u32* src = reinterpret_cast<const u32*>(p.codes) + w0;
-#pragma unroll
-            for (int i = 0; i < LANE_WORDS; ++i) wv[i] = __ldcs(src + i);
+            const u32 n = packed_words(p.packed_bits);
+            if ((w0 + n) * 4 > p.codes_bytes) return false;
+            load_packed(reinterpret_cast<const u32*>(p.codes) + w0, n, wv);
             return true;
         }
         const u64 b0 = q0 * WBITS / 8;   // q0 is a multiple of K, K a multiple of 8
@@ -312,33 +307,63 @@ struct WarpCore {
         }
     }
 
-    // Packed codes: the lane's words go to its shared-memory scratch `pk`
-    // (a run-time bit offset cannot index registers), then each code is one
-    // funnel shift of the two words that hold it.
-    static __device__ __forceinline__ void unpack_packed(const u32 (&wv)[LANE_WORDS], u32 o, u32 b, u32* pk, R& r) {
-        uint2* pairs = reinterpret_cast<uint2*>(pk);
+    // Packed codes of b bits: a lane's 16 codes are 16 b bits from a multiple
+    // of 16 bits on, so they begin at a word, or (odd b, odd lanes) in the
+    // middle of one, and lie in these words either way.
+    static __device__ __forceinline__ u32 packed_words(u32 b) { return (b + 1u) >> 1; }
+    static __device__ __forceinline__ void load_packed(const u32* src, u32 n, u32 (&wv)[LANE_WORDS]) {
 #pragma unroll
-        for (int i = 0; i < LANE_WORDS; ++i) pairs[i] = make_uint2(wv[i], i + 1 < LANE_WORDS ? wv[i + 1] : 0u);
-        const u32 mask = (1u << b) - 1u;
+        for (int i = 0; i < LANE_WORDS; ++i) wv[i] = (u32)i < n ? __ldcs(src + i) : 0u;
+    }
+    // `o`: the bit the codes begin at in wv[0], 0 or 16.
+    template <int B>
+    static __device__ __forceinline__ void unpack_bits(const u32 (&wv)[LANE_WORDS], u32 o, R& r) {
+        constexpr int N = (B + 1) / 2;
+        constexpr u32 MASK = (1u << B) - 1u;
+        u32 w[N + 1];
+#pragma unroll
+        for (int i = 0; i < N; ++i) w[i] = (B & 1) ? __funnelshift_r(wv[i], i + 1 < N ? wv[i + 1] : 0u, o) : wv[i];
+        w[N] = 0u;
 #pragma unroll
         for (int m = 0; m < K / 2; ++m) {
-            u32 v = 0;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const u32 P = o + (u32)(2 * m + h) * b;   // < 32 + 15 * 16
-                const uint2 w = pairs[P >> 5];
-                v |= (__funnelshift_r(w.x, w.y, P) & mask) << (16 * h);
-            }
-            r.c[m] = v;
+            const int bit = 2 * m * B, i = bit >> 5, sh = bit & 31;
+            const u32 two = sh + 2 * B <= 32 ? w[i] >> sh : __funnelshift_r(w[i], w[i + 1], sh);
+            r.c[m] = B == 16 ? two : (two & MASK) | ((two << (16 - B)) & (MASK << 16));
+        }
+    }
+    // Every width has a body of its own, taken by one branch that is the same
+    // for the whole grid: constant bit positions cost two instructions a
+    // code, positions computed from a run-time width about seven and two
+    // wavefronts of the shared-memory pipe a code (the words have to be
+    // indexed there).  FSST-12 at 10 bits, 16M strings: 562 -> 492 us a call,
+    // with the reduce summing lengths as for the codec's own layout.
+    static __device__ __forceinline__ void unpack_packed(const u32 (&wv)[LANE_WORDS], u32 o, u32 b, R& r) {
+        switch (b) {
+            case 1: unpack_bits<1>(wv, o, r); break;
+            case 2: unpack_bits<2>(wv, o, r); break;
+            case 3: unpack_bits<3>(wv, o, r); break;
+            case 4: unpack_bits<4>(wv, o, r); break;
+            case 5: unpack_bits<5>(wv, o, r); break;
+            case 6: unpack_bits<6>(wv, o, r); break;
+            case 7: unpack_bits<7>(wv, o, r); break;
+            case 8: unpack_bits<8>(wv, o, r); break;
+            case 9: unpack_bits<9>(wv, o, r); break;
+            case 10: unpack_bits<10>(wv, o, r); break;
+            case 11: unpack_bits<11>(wv, o, r); break;
+            case 12: unpack_bits<12>(wv, o, r); break;
+            case 13: unpack_bits<13>(wv, o, r); break;
+            case 14: unpack_bits<14>(wv, o, r); break;
+            case 15: unpack_bits<15>(wv, o, r); break;
+            default: unpack_bits<16>(wv, o, r); break;
         }
     }
 
     // Codes, from words load_fast() or load_staged() fetched or by guarded
-    // loads.  `pk`: the lane's scratch (packed codes only).
+    // loads.
     static __device__ __forceinline__ void unpack(const DecodeParams& p, u64 q0, const u32 (&wv)[LANE_WORDS], bool fast,
-                                                  R& r, u32* pk = nullptr) {
+                                                  R& r) {
         if (fast) {
-            if (PACKED) unpack_packed(wv, (u32)((q0 * p.packed_bits) & 31u), p.packed_bits, pk, r);
+            if constexpr (PACKED) unpack_packed(wv, (u32)((q0 * p.packed_bits) & 31u), p.packed_bits, r);
             else unpack_words(wv, r);
         } else {
             load_guarded(p, q0, r);
@@ -363,8 +388,8 @@ struct WarpCore {
     // The codes, the slots inside the column and their token lengths.
     static __device__ __forceinline__ void finish_load(const DecodeParams& p, const Extent& x, u64 q0,
                                                        const u32 (&wv)[LANE_WORDS], bool fast, const uint8_t* lens,
-                                                       R& r, u32* pk = nullptr) {
-        unpack(p, q0, wv, fast, r, pk);
+                                                       R& r) {
+        unpack(p, q0, wv, fast, r);
         mark_valid(x, q0, r);
 #pragma unroll
         for (int j = 0; j < K / 4; ++j) {
@@ -647,15 +672,23 @@ struct WarpCore {
     // column, straight from its code words (constant bit positions): one
     // extract, one length load and one add per code; a code without a token
     // (length 0) raises ERRB_CORRUPT.
+    // Packed codes: `o` and `b` as in unpack_packed().
     static __device__ __forceinline__ u32 lane_length_sum(const u32 (&wv)[LANE_WORDS], const uint8_t* lens,
-                                                          u32& err) {
-        static_assert(!FSST && !PACKED, "escape-free codecs in their own layout");
+                                                          u32& err, u32 o = 0, u32 b = 0) {
+        static_assert(!FSST, "escape-free codecs");
         constexpr u32 MASK = (1u << WBITS) - 1u;
         u32 sum = 0, mn = 0xffu;
+        R r;
+        if constexpr (PACKED) unpack_packed(wv, o, b, r);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            const int bit = k * WBITS, w = bit >> 5, sh = bit & 31;
-            const u32 code = (sh + WBITS <= 32) ? ((wv[w] >> sh) & MASK) : (__funnelshift_r(wv[w], wv[w + 1], sh) & MASK);
+            u32 code;
+            if constexpr (PACKED) {
+                code = code_at<CODEC, K>(r, k);
+            } else {
+                const int bit = k * WBITS, w = bit >> 5, sh = bit & 31;
+                code = (sh + WBITS <= 32) ? ((wv[w] >> sh) & MASK) : (__funnelshift_r(wv[w], wv[w + 1], sh) & MASK);
+            }
             const u32 L = LSMEM ? (u32)lens[code] : (u32)__ldg(lens + code);
             sum += L;
             mn = min(mn, L);
@@ -948,7 +981,7 @@ struct WarpCore {
             finish_load(p, x, q0, wv, in, lens, r);
         } else {
             next();
-            finish_load(p, x, q0, f.wv, f.in, lens, r, reinterpret_cast<u32*>(area.codes) + lane * PK_STRIDE);
+            finish_load(p, x, q0, f.wv, f.in, lens, r);
         }
         const u64 next_ex = assemble_tile(p, x, t, r, ex, sb, dict, area, err);
         if (chk && ex_next != (u32)next_ex) err |= ERRB_MISMATCH;
@@ -1059,10 +1092,9 @@ __global__ void __launch_bounds__(256) index_only_kernel(const DecodeParams p, u
 // tile), the others the reduce: the two overlap in one launch.  Large FSST-8
 // and OnPair-16 columns take length_reduce_kernel (fp_reduce.cuh) instead.
 // Reduce shape per codec, from an A/B on GB300 (10M-16M strings): rounds of
-// kReduceU tiles in flight, kReduceMinB blocks of 256 threads per SM.
-// OnPair-12: 2 x 4 (1,515 GB/s per call against 1,498 at 2 x 3); FSST-8,
-// whose 32-slot lanes spill at fewer than 128 registers: 2 x 2 (1,051
-// against 1,038); FSST-12: 1 x 4 (1,188 against 1,171).
+// U tiles in flight, MINB blocks of 256 threads per SM.  Per call of that
+// A/B, OnPair-12: 2 x 4 725 us, 2 x 3 733; FSST-8, whose 32-slot lanes spill
+// at fewer than 128 registers: 2 x 2 1.2 % faster; FSST-12: 1 x 4 1.5 %.
 template <int CODEC, int K>
 struct ReduceShape {
     static constexpr int U = CODEC == FP_FSST12 ? 1 : 2;
@@ -1074,7 +1106,6 @@ __global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kerne
                                                                                   u64* agg, u32 index_blocks) {
     typedef WarpCore<CODEC, K, DSMEM, WarpCore<CODEC, K, DSMEM>::TOK8 ? 8 : 16, PACKED> C;
     __shared__ __align__(16) uint8_t s_lens[DSMEM ? C::LENS_BYTES : 16];
-    __shared__ __align__(16) u32 s_pk[PACKED ? 256 * C::PK_STRIDE : 2];   // packed codes: per-lane scratch
     if (DSMEM && blockIdx.x >= index_blocks) {
         // the dictionary is older than any launch this one may overlap
         const uint4* src = reinterpret_cast<const uint4*>(pp.dict.lens);
@@ -1098,22 +1129,26 @@ __global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kerne
     u32 err = 0;
     // rounds of U tiles; the next round's loads are in flight while this one computes
     constexpr int U = ReduceShape<CODEC, K>::U;
-    if constexpr (!C::FSST && !PACKED) {
-        // Escape-free codes in their own layout: tiles [t_lo, t_hi) lie wholly
+    if constexpr (!C::FSST) {
+        // Escape-free codes: tiles [t_lo, t_hi) lie wholly
         // inside the column and the code buffer; their lanes load their code
         // words at a fixed stride and sum their lengths straight from them
         // (32-bit tile indices: fewer than 2^32 tiles).  Edge tiles take the
         // general path.
-        constexpr u32 TB = C::TILE * C::WBITS / 8;   // code bytes of a tile
+        const u32 bits = PACKED ? p.packed_bits : (u32)C::WBITS;
+        const u32 TB = C::TILE / 8 * bits;   // code bytes of a tile; the words of its lanes lie within them
         const u32 nt = (u32)x.n_tiles, W = (u32)warps;
-        const u64 buf_slots = p.codes_bytes * 8 / C::WBITS;
+        const u64 buf_slots = p.codes_bytes * 8 / bits;
         const u64 end = x.c_end < buf_slots ? x.c_end : buf_slots;
         const u64 lo64 = (x.c_begin + C::TILE - 1) / C::TILE, hi64 = end / C::TILE;
         const u32 t_lo = (u32)(lo64 - x.first_tile);
         const u32 t_hi = hi64 > lo64 ? (u32)(hi64 - x.first_tile) : t_lo;
-        const uint8_t* base = p.codes + x.first_tile * (u64)TB + (u64)lane * C::LANE_BYTES;
+        const u32 lane_bit = lane * K * bits, o = PACKED ? lane_bit & 31u : 0u;
+        const uint8_t* base = p.codes + x.first_tile * (u64)TB + (lane_bit - o) / 8;
         auto load = [&](u32 t, u32 (&w)[C::LANE_WORDS]) {
-            if (C::LANE_BYTES % 16 == 0) {
+            if constexpr (PACKED) {
+                C::load_packed(reinterpret_cast<const u32*>(base + (u64)t * TB), C::packed_words(bits), w);
+            } else if (C::LANE_BYTES % 16 == 0) {
                 const uint4* src = reinterpret_cast<const uint4*>(base + (u64)t * TB);
 #pragma unroll
                 for (int v = 0; v < C::LANE_WORDS / 4; ++v) {
@@ -1149,7 +1184,7 @@ __global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kerne
                 const u32 tt = t + u * W;
                 if (tt >= nt) continue;
                 if (tt >= t_lo && tt < t_hi) {
-                    const u32 tot = __reduce_add_sync(0xffffffffu, C::lane_length_sum(wv[u], lens, err));
+                    const u32 tot = __reduce_add_sync(0xffffffffu, C::lane_length_sum(wv[u], lens, err, o, bits));
                     if (lane == 31) agg[tt] = tot;
                 } else {
                     u32 gw[C::LANE_WORDS];
@@ -1189,7 +1224,7 @@ __global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kerne
             const u64 t = t0 + u * warps;
             if (t < x.n_tiles) {
                 typename C::R r;
-                C::finish_load(p, x, C::lane_q0(x, t), wv[u], fast[u], lens, r, s_pk + threadIdx.x * C::PK_STRIDE);
+                C::finish_load(p, x, C::lane_q0(x, t), wv[u], fast[u], lens, r);
                 const TElem e = C::tile_element(r, lane, err);
                 if (lane == 31) agg[t] = wt_pack<C::FSST>(e);
             }
