@@ -1,21 +1,22 @@
 // Batched decode: many column chunks (mixed codecs, one dictionary each) in
-// one persistent launch, replayed from a CUDA graph.
+// a fixed set of launches, replayed from a CUDA graph.
 //
-// Work queue.  Chunks are grouped by codec into three queues; a queue's
-// tickets run over the tiles of all its chunks (chunk after chunk), and a
-// table maps a ticket to its chunk.  Every block runs the decode pipeline of
-// fp_decoder.cuh on one queue until it is exhausted, then moves on to the
-// next queue, so a block never idles while any queue has tiles.  Blocks are
-// spread over the queues in proportion to their code slots at the start.
+// Work queues.  Chunks are grouped by codec into four queues.  The block
+// pipeline runs one persistent launch: a queue's tickets run over the tiles of
+// all its chunks (chunk after chunk), a table maps a ticket to its chunk, and
+// a block moves on to the next queue when one is exhausted; blocks are spread
+// over the queues in proportion to their code slots at the start.  Warp tiles
+// run a reduce, a tile scan and a decode over all queues; the staged
+// configuration (the default) a reduce and a decode per codec.
 //
 // Per-chunk state.  A chunk's code buffer is tiled whole (tile u = slots
 // [u*T, (u+1)*T)); each chunk has its own look-back words, tile -> string
 // index, data-error word and decoded size.  The decode block copies the
 // chunk's record (SlotSrc) into its ring slot with the tile's inputs, so
 // consecutive tiles of one block may belong to different chunks and codecs.
-// Dictionaries are read through the L1 cache here (a copy into shared memory
+// Dictionaries are read through the L1 cache there (a copy into shared memory
 // would have to be repeated at every chunk change); the staged configuration
-// below cuts the chunks into units so that it pays.
+// cuts the chunks into units so that it pays.
 //
 // Autotuning.  The tile shape (code slots per thread for each codec) and
 // the blocks per SM are compiled or launch-time choices; fp_plan_create
@@ -1066,7 +1067,7 @@ fp_status plan_create(const fp_chunk* chunks, uint32_t n, int force_cfg, const c
 namespace fp {
 
 // Staged units: the fastest configuration on every mixed batch measured (256
-// chunks of 4 KB - 16 MB: 471 us against 602 us for warp tiles through L1; 60
+// chunks of 4 KB - 16 MB: 465 us against 602 us for warp tiles through L1; 60
 // chunks up to 1 MB: 48 against 55; 16 up to 4 MB: 37 against 57).
 int batch_config_default() { return 5; }
 

@@ -50,17 +50,15 @@ const Variant* variant_get(int codec, int v) {
 
 // Defaults chosen by measurement on GB300 (synthetic columns, every variant
 // timed at 30k..10M strings): warp tiles for every codec, one block of 16
-// warps per SM for large columns.  The one-block shapes run the same code
-// with the same registers and warps per SM as two blocks of 8 warps, with one
-// copy of the dictionary per SM instead of two; they were faster for every
-// codec (10M strings: OnPair-12 1446 vs 1342 GB/s, FSST-8 963 vs 902,
-// OnPair-16 1029 vs 990).  OnPair-12 below 2^23 slots reads the dictionary
-// through L1 (20 warps; staging it per block does not pay: 637 vs 613 GB/s
-// at 300k strings); FSST-8 below 2^22 slots uses 16-slot lanes.  The OnPair
-// codecs come in both read widths (split read W = 8, whole entries W = 16);
-// the dictionary's width picks between them.  FSST-12 stages its 32 KiB
-// table in shared memory at every size (16M strings: 1,134 GB/s with 32-slot
-// lanes, 1,113 with 16; 300k strings: 368 against 337 through L1).
+// warps per SM for large columns, with the dictionary (OnPair-16: its
+// lengths) in shared memory: OnPair-12, 10M strings, 583 us a call against 797
+// with the table read through L1; OnPair-16, 2M strings, 174 against 198 for
+// blocks of 8 warps; FSST-8, 16M strings, 529 with 32-slot lanes against 562
+// for blocks of 8 warps and 698 with 16-slot lanes; FSST-12, 20k documents, 99
+// with 32-slot lanes, 106 with 16, 130 through L1.  The smaller shapes below
+// 2^23 and 2^22 slots are the built-in rule where no tuned one is loaded.  The
+// OnPair codecs come in both read widths (split read W = 8, whole entries W =
+// 16); the dictionary's width picks between them.
 //
 // Below 2^17 slots (256 tiles of 512: one to a warp of 16 blocks) the whole
 // column goes to one cluster in one launch: 8.7-9.5 us a call back to back
