@@ -67,7 +67,7 @@ SERVE_WORKLOADS = {
 }
 METRIC = "decoded GB/s (single-column decode, inputs resident in HBM)"
 SERVE_METRIC = "served decode: aggregate decoded GB/s at the offered load, with p50/p99 latency"
-SERVE_DEFAULT_CONFIG = 5   # the library's default batch configuration (staged units)
+SERVE_DEFAULT_CONFIG = -1   # the library chooses a batch configuration for each wave, 4 or 5
 BATCH_METRIC = "decoded GB/s (batched decode of many chunks, inputs resident in HBM)"
 L2_BYTES = 126 * 1024 * 1024
 
@@ -1384,7 +1384,7 @@ def run_served(args, rank, world, local_rank):
         "clocks": clocks,
         # per wave: index pass [+ reduce + tile scan] + the persistent decode kernel; staged: a reduce and a
         # decode per codec in the wave, counted here for waves of one codec (two more for each further one)
-        "gpu_launches": batch_launches(fp.batch_config_info(serve_cfg), 1) * waves,
+        "gpu_launches": batch_launches(fp.batch_config_info(serve_cfg if serve_cfg >= 0 else 4), 1) * waves,
     }
     line.update(extra)
     if "e2e" not in line:

@@ -449,7 +449,7 @@ typedef struct fp_serve_config {
     uint32_t n_streams;         /* waves in flight at once (0 = 4) */
     uint32_t max_wave;          /* requests per wave (0 = 256) */
     int32_t batch_config;       /* batch configuration of the waves (fp_batch_config_info); negative:
-                                   the library's default */
+                                   chosen for each wave by its size */
     uint32_t reserved;
 } fp_serve_config;
 

@@ -7,7 +7,7 @@
 // a block moves on to the next queue when one is exhausted; blocks are spread
 // over the queues in proportion to their code slots at the start.  Warp tiles
 // run a reduce, a tile scan and a decode over all queues; the staged
-// configuration (the default) a reduce and a decode per codec.
+// configuration a reduce and a decode per codec.
 //
 // Per-chunk state.  A chunk's code buffer is tiled whole (tile u = slots
 // [u*T, (u+1)*T)); each chunk has its own look-back words, tile -> string
@@ -1066,10 +1066,18 @@ fp_status plan_create(const fp_chunk* chunks, uint32_t n, int force_cfg, const c
 
 namespace fp {
 
-// Staged units: the fastest configuration on every mixed batch measured (256
-// chunks of 4 KB - 16 MB: 465 us against 602 us for warp tiles through L1; 60
-// chunks up to 1 MB: 48 against 55; 16 up to 4 MB: 37 against 57).
-int batch_config_default() { return 5; }
+// Staged units are the fastest configuration on the device for every mixed
+// batch measured (256 chunks of 4 KB - 16 MB: 465 us against 602 us for warp
+// tiles through L1; 60 chunks up to 1 MB: 48 against 55; 16 up to 4 MB: 37
+// against 57), but a wave is enqueued launch by launch, up to ten instead of
+// four (about 2.5 us of the host each).  32 requests, 110 MB decoded, in three
+// waves: 1,507 us with warp tiles, 1,559 staged; at the gain of 0.12 us per MB
+// the staged launches pay from about 200 MB on.
+int wave_config(const fp_chunk* chunks, uint32_t n) {
+    uint64_t bytes = 0;
+    for (uint32_t i = 0; i < n; ++i) bytes += chunks[i].out_capacity;
+    return bytes >= (192ull << 20) ? 5 : 4;
+}
 
 fp_status wave_init(WaveBuffers& W, uint32_t cap_chunks) {
     int dev = 0;

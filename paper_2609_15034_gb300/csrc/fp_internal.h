@@ -228,7 +228,7 @@ void wave_free(WaveBuffers& W);
 // per-chunk results into W.h_status / W.h_total.  The previous wave of W
 // must have completed (its staging is reused).
 fp_status wave_launch(WaveBuffers& W, const fp_chunk* chunks, uint32_t n, int config, cudaStream_t stream);
-int batch_config_default();
+int wave_config(const fp_chunk* chunks, uint32_t n);
 
 // Host helpers (fp_api.cu).
 fp_status fail(fp_status st, const char* fmt, ...);          // sets fp_last_error()

@@ -19,6 +19,8 @@
 //     decoded size and the host times of submission, admission and
 //     completion.
 // Requests are admitted in arrival order (no overtaking).
+#include <sys/prctl.h>
+
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -99,6 +101,7 @@ struct Slot {
     uint32_t refs = 0;            // admitted requests not yet completed
     uint64_t lru = 0;
     cudaEvent_t ready = nullptr;  // recorded after the upload into the slot
+    bool resident = false;        // that upload is known to have completed
     fp_dict view{};
 };
 
@@ -127,7 +130,7 @@ struct Lane {
 struct fp_server {
     fp_serve_config cfg{};
     int device = 0;
-    int config = 0;
+    int config = 0;   // of every wave; negative: by the wave's size
     char* d_arena = nullptr;
     Arena arena;
     char* d_dicts = nullptr;
@@ -239,8 +242,15 @@ void lane_launch(fp_server* S, Lane& L) {
                 if (e == cudaSuccess)
                     e = cudaMemcpyAsync(sl.view.d_lens, hd.h_lens, hd.lens_bytes, cudaMemcpyHostToDevice, L.s);
                 if (e == cudaSuccess) e = cudaEventRecord(sl.ready, L.s);
+                sl.resident = false;
+            } else if (!sl.resident) {
+                // a stream waits only for an upload that is not known to be done:
+                // a wave of 30 requests issued 30 waits with the queue locked
+                e = cudaEventQuery(sl.ready);
+                if (e == cudaSuccess) sl.resident = true;
+                else if (e == cudaErrorNotReady) e = cudaStreamWaitEvent(L.s, sl.ready, 0);
             } else {
-                e = cudaStreamWaitEvent(L.s, sl.ready, 0);
+                e = cudaSuccess;
             }
             if (e != cudaSuccess) {
                 // the device refused the dictionary's upload: fail this request (a dead context
@@ -286,7 +296,8 @@ void lane_launch(fp_server* S, Lane& L) {
         }
     }
     if (L.reqs.empty()) return;
-    fp_status stt = wave_launch(L.W, chunks.data(), (uint32_t)chunks.size(), S->config, L.s);
+    const int config = S->config >= 0 ? S->config : wave_config(chunks.data(), (uint32_t)chunks.size());
+    fp_status stt = wave_launch(L.W, chunks.data(), (uint32_t)chunks.size(), config, L.s);
     cudaError_t e = cudaSuccess;
     if (stt == FP_OK) e = cudaEventRecord(L.ev, L.s);
     if (stt != FP_OK || e != cudaSuccess) {
@@ -337,6 +348,9 @@ void lane_fail(fp_server* S, Lane& L, cudaError_t e) {
 
 void scheduler(fp_server* S) {
     cudaSetDevice(S->device);
+    // this thread's sleeps end within a microsecond of their time: with the
+    // default slack of 50 us the 20 us between two looks at the lanes took 70
+    prctl(PR_SET_TIMERSLACK, 1000UL, 0UL, 0UL, 0UL);
     for (;;) {
         bool stopping = false;
         {
@@ -417,7 +431,7 @@ fp_status fp_serve_create(const fp_serve_config* cfg_in, fp_server** out) {
         return fail(FP_ERR_ARG, "serve configuration out of range");
     fp_server* S = new fp_server();
     S->cfg = cfg;
-    S->config = cfg.batch_config >= 0 ? cfg.batch_config : batch_config_default();
+    S->config = cfg.batch_config;
     if (S->config >= fp_batch_config_count()) {
         delete S;
         return fail(FP_ERR_ARG, "batch configuration %d out of range", cfg.batch_config);
