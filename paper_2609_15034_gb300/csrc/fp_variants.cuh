@@ -86,7 +86,7 @@ Variant make_cluster_variant() {
 // shared-memory scratch for the code words.
 template <int CODEC, bool DSMEM, int NW>
 Variant make_packed_variant() {
-    constexpr int K = 16, W = (CODEC == FP_FSST12) ? 8 : 16;
+    constexpr int K = CODEC == FP_FSST12 ? 32 : 16, W = CODEC == FP_FSST12 ? 8 : 16;
     typedef WarpCore<CODEC, K, DSMEM, W, true, true> C;
     Variant v{};
     v.threads = NW * 32;

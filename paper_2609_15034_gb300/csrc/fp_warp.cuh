@@ -152,9 +152,8 @@ struct WarpCore {
     static constexpr int TILE = 32 * K;
     static constexpr int WBITS = (CODEC == FP_ONPAIR16) ? 16 : (W12 ? 12 : 8);
     static constexpr int LANE_BYTES = K * WBITS / 8;   // code bytes of one lane
-    // words a lane loads: its code bytes; for packed codes up to 16 codes of
-    // 16 bits, which begin at a word or in the middle of one (packed_words())
-    static constexpr int LANE_WORDS = PACKED ? K / 2 : LANE_BYTES / 4;
+    // words a lane loads: its code bytes, or (packed codes) at most as many
+    static constexpr int LANE_WORDS = LANE_BYTES / 4;
     // entries of the table (a staged table, or the global planes)
     static constexpr int kTable = (CODEC == FP_FSST8) ? 256 : (CODEC == FP_ONPAIR16 ? 65536 : 4096);
     // FSST-8 with a staged table: the symbols, then the 256 literal bytes as
@@ -165,7 +164,10 @@ struct WarpCore {
     // tokens of 7.5 bytes: 3.8 KB; 1,024 FSST symbols: 4.6 KB); less where
     // the dictionary is read through L1, which shares the SM's memory.
     static constexpr int CAP = DSMEM ? 6144 : 4096;
-    static constexpr int TILE_BYTES = TILE * WBITS / 8;   // code bytes of a tile
+    static constexpr int TILE_BYTES = TILE * WBITS / 8;   // code bytes of a tile, at most
+    static __device__ __forceinline__ u32 tile_bytes(const DecodeParams& p) {
+        return PACKED ? TILE / 8 * p.packed_bits : (u32)TILE_BYTES;   // a multiple of 16
+    }
     // The next tile's codes come by a bulk copy into the warp's area (32-slot
     // lanes), or into registers.  The copy frees 8 to 12 registers and
     // writes each line once where lanes 32 or 48 bytes apart touch it several
@@ -183,7 +185,7 @@ struct WarpCore {
     static_assert(LANE_BYTES % 8 == 0, "lane code bytes are read in 8-byte words");
     static_assert(W == 16 || W == 8, "read width");
     static_assert(!TOK8 || W == 8, "FSST entries are 8 bytes");
-    static_assert(!PACKED || (!FSST && K == 16), "packed codes: escape-free codecs, 16 slots per lane");
+    static_assert(!PACKED || (!FSST && K >= 16), "packed codes: escape-free codecs, 16 or 32 slots per lane");
 
     static __device__ __forceinline__ u32 full_mask() { return K == 32 ? 0xffffffffu : ((1u << K) - 1u); }
 
@@ -235,7 +237,15 @@ struct WarpCore {
     }
 
     // The same words from the tile's bulk-copied code bytes.
-    static __device__ __forceinline__ void load_staged(const uint4* codes, u32 lane, u32 (&wv)[LANE_WORDS]) {
+    static __device__ __forceinline__ void load_staged(const DecodeParams& p, const uint4* codes, u32 lane,
+                                                       u32 (&wv)[LANE_WORDS]) {
+        if (PACKED) {
+            // words b apart over the lanes: at most 8 lanes of a load share a bank (b = 8), 2 at 10 bits
+            const u32* src = reinterpret_cast<const u32*>(codes) + lane * p.packed_bits;
+#pragma unroll
+            for (int i = 0; i < LANE_WORDS; ++i) wv[i] = (u32)i < p.packed_bits ? src[i] : 0u;
+            return;
+        }
 #pragma unroll
         for (int v = 0; v < LANE_BYTES / 16; ++v) {
             const uint4 a = codes[lane * (LANE_BYTES / 16) + v];
@@ -307,10 +317,10 @@ struct WarpCore {
         }
     }
 
-    // Packed codes of b bits: a lane's 16 codes are 16 b bits from a multiple
-    // of 16 bits on, so they begin at a word, or (odd b, odd lanes) in the
-    // middle of one, and lie in these words either way.
-    static __device__ __forceinline__ u32 packed_words(u32 b) { return (b + 1u) >> 1; }
+    // Packed codes of b bits: 32 of them are b words.  A lane's 16 are 16 b bits
+    // from a multiple of 16 bits on, so they begin at a word, or (odd b, odd
+    // lanes) in the middle of one, and lie in these words either way.
+    static __device__ __forceinline__ u32 packed_words(u32 b) { return K == 32 ? b : (b + 1u) >> 1; }
     static __device__ __forceinline__ void load_packed(const u32* src, u32 n, u32 (&wv)[LANE_WORDS]) {
 #pragma unroll
         for (int i = 0; i < LANE_WORDS; ++i) wv[i] = (u32)i < n ? __ldcs(src + i) : 0u;
@@ -318,11 +328,11 @@ struct WarpCore {
     // `o`: the bit the codes begin at in wv[0], 0 or 16.
     template <int B>
     static __device__ __forceinline__ void unpack_bits(const u32 (&wv)[LANE_WORDS], u32 o, R& r) {
-        constexpr int N = (B + 1) / 2;
+        constexpr int N = (K * B + 31) / 32;
         constexpr u32 MASK = (1u << B) - 1u;
         u32 w[N + 1];
 #pragma unroll
-        for (int i = 0; i < N; ++i) w[i] = (B & 1) ? __funnelshift_r(wv[i], i + 1 < N ? wv[i + 1] : 0u, o) : wv[i];
+        for (int i = 0; i < N; ++i) w[i] = (K == 16 && (B & 1)) ? __funnelshift_r(wv[i], i + 1 < N ? wv[i + 1] : 0u, o) : wv[i];
         w[N] = 0u;
 #pragma unroll
         for (int m = 0; m < K / 2; ++m) {
@@ -330,6 +340,11 @@ struct WarpCore {
             const u32 two = sh + 2 * B <= 32 ? w[i] >> sh : __funnelshift_r(w[i], w[i + 1], sh);
             r.c[m] = B == 16 ? two : (two & MASK) | ((two << (16 - B)) & (MASK << 16));
         }
+    }
+    // (a width above the codec's own is refused by the host)
+    template <int B>
+    static __device__ __forceinline__ void unpack_width(const u32 (&wv)[LANE_WORDS], u32 o, R& r) {
+        unpack_bits<B <= WBITS ? B : WBITS>(wv, o, r);
     }
     // Every width has a body of its own, taken by one branch that is the same
     // for the whole grid: constant bit positions cost two instructions a
@@ -339,22 +354,22 @@ struct WarpCore {
     // with the reduce summing lengths as for the codec's own layout.
     static __device__ __forceinline__ void unpack_packed(const u32 (&wv)[LANE_WORDS], u32 o, u32 b, R& r) {
         switch (b) {
-            case 1: unpack_bits<1>(wv, o, r); break;
-            case 2: unpack_bits<2>(wv, o, r); break;
-            case 3: unpack_bits<3>(wv, o, r); break;
-            case 4: unpack_bits<4>(wv, o, r); break;
-            case 5: unpack_bits<5>(wv, o, r); break;
-            case 6: unpack_bits<6>(wv, o, r); break;
-            case 7: unpack_bits<7>(wv, o, r); break;
-            case 8: unpack_bits<8>(wv, o, r); break;
-            case 9: unpack_bits<9>(wv, o, r); break;
-            case 10: unpack_bits<10>(wv, o, r); break;
-            case 11: unpack_bits<11>(wv, o, r); break;
-            case 12: unpack_bits<12>(wv, o, r); break;
-            case 13: unpack_bits<13>(wv, o, r); break;
-            case 14: unpack_bits<14>(wv, o, r); break;
-            case 15: unpack_bits<15>(wv, o, r); break;
-            default: unpack_bits<16>(wv, o, r); break;
+            case 1: unpack_width<1>(wv, o, r); break;
+            case 2: unpack_width<2>(wv, o, r); break;
+            case 3: unpack_width<3>(wv, o, r); break;
+            case 4: unpack_width<4>(wv, o, r); break;
+            case 5: unpack_width<5>(wv, o, r); break;
+            case 6: unpack_width<6>(wv, o, r); break;
+            case 7: unpack_width<7>(wv, o, r); break;
+            case 8: unpack_width<8>(wv, o, r); break;
+            case 9: unpack_width<9>(wv, o, r); break;
+            case 10: unpack_width<10>(wv, o, r); break;
+            case 11: unpack_width<11>(wv, o, r); break;
+            case 12: unpack_width<12>(wv, o, r); break;
+            case 13: unpack_width<13>(wv, o, r); break;
+            case 14: unpack_width<14>(wv, o, r); break;
+            case 15: unpack_width<15>(wv, o, r); break;
+            default: unpack_width<16>(wv, o, r); break;
         }
     }
 
@@ -736,11 +751,12 @@ struct WarpCore {
     static __device__ __forceinline__ void fetch_codes(const DecodeParams& p, const Extent& x, u64 t, Area& area,
                                                        const CodeBar& cb, Fetch& f) {
         if constexpr (BULK_CODES) {
-            const u64 b0 = (x.first_tile + t) * TILE_BYTES;   // a multiple of 16, as TILE_BYTES is
-            f.in = b0 + TILE_BYTES <= p.codes_bytes;
+            const u32 tb = tile_bytes(p);
+            const u64 b0 = (x.first_tile + t) * tb;   // a multiple of 16, as tb is
+            f.in = b0 + tb <= p.codes_bytes;
             if (f.in && (threadIdx.x & 31u) == 0u) {
-                mbar_expect_tx(cb.bar, (u32)TILE_BYTES);
-                bulk_g2s(area.codes, p.codes + b0, (u32)TILE_BYTES, cb.bar);
+                mbar_expect_tx(cb.bar, tb);
+                bulk_g2s(area.codes, p.codes + b0, tb, cb.bar);
                 mbar_arrive(cb.bar);
             }
         } else {
@@ -974,7 +990,7 @@ struct WarpCore {
             if (in) {
                 mbar_wait(cb.bar, cb.phase, p.ws);
                 cb.phase ^= 1u;
-                load_staged(area.codes, lane, wv);
+                load_staged(p, area.codes, lane, wv);
             }
             __syncwarp();   // the codes have left the area
             next();
@@ -1136,7 +1152,7 @@ __global__ void __launch_bounds__(256, ReduceShape<CODEC, K>::MINB) reduce_kerne
         // (32-bit tile indices: fewer than 2^32 tiles).  Edge tiles take the
         // general path.
         const u32 bits = PACKED ? p.packed_bits : (u32)C::WBITS;
-        const u32 TB = C::TILE / 8 * bits;   // code bytes of a tile; the words of its lanes lie within them
+        const u32 TB = C::tile_bytes(p);   // the words of its lanes lie within them
         const u32 nt = (u32)x.n_tiles, W = (u32)warps;
         const u64 buf_slots = p.codes_bytes * 8 / bits;
         const u64 end = x.c_end < buf_slots ? x.c_end : buf_slots;

@@ -11,13 +11,13 @@ from test_gpu_packed import fp, pack_bits, run, small_dict  # noqa: F401  (fp: t
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("b", range(1, 17))
-def test_width(fp, b):  # noqa: F811
-    codec = synth.ONPAIR16 if b > 12 or b % 2 else (synth.ONPAIR12 if b % 4 else synth.FSST12)
+@pytest.mark.parametrize("codec,b", [(c, b) for c in (synth.ONPAIR16, synth.ONPAIR12, synth.FSST12)
+                                     for b in range(1, synth.CODE_BITS[c] + 1)])
+def test_width(fp, codec, b):  # noqa: F811
     rng = np.random.default_rng(900 + b)
     n_entries = min(1 << b, 5000 if b > 12 else 4096)
     d = small_dict(codec, n_entries, rng)
-    for n in (16, 31, 512, 513, 5 * 512 + 16, 8192 + 496):
+    for n in (16, 31, 512, 1024, 1025, 5 * 512 + 16, 8192 + 496):
         codes = rng.integers(0, n_entries, n).astype(np.uint32)
         codes[-16:] = n_entries - 1
         stream = pack_bits(codes, b)   # ends with the last code's byte: no padding to a word
