@@ -82,8 +82,7 @@ Variant make_cluster_variant() {
     return v;
 }
 
-// Packed codes (run-time width): the warp-tile decoder with a per-lane
-// shared-memory scratch for the code words.
+// Packed codes (run-time width): the warp-tile decoder, a body per width.
 template <int CODEC, bool DSMEM, int NW>
 Variant make_packed_variant() {
     constexpr int K = CODEC == FP_FSST12 ? 32 : 16, W = CODEC == FP_FSST12 ? 8 : 16;

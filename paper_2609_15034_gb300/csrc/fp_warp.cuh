@@ -125,7 +125,7 @@ struct StageWriter {
 template <int K, int CAP, int CODE_BYTES>
 struct WarpArea {
     uint4 stage[CAP / 16 + 1];
-    // code bytes of the tile to decode next (bulk copy), or the unpack's scratch (packed codes)
+    // code bytes of the tile to decode next (bulk copy)
     uint4 codes[CODE_BYTES ? CODE_BYTES / 16 : 1];
     u32 pre[K / 4][32];     // tile-relative output offset of slot 4m of each lane
     u32 contrib[K / 4][32]; // bytes each slot produced, one byte per slot
