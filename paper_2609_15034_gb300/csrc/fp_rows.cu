@@ -192,12 +192,14 @@ __global__ void __launch_bounds__(kRowBlock) rows_gather_kernel(const RowsArgs a
     const u32 m = a.n_rows, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     u32* const wv = s_v[warp];
     u32* const wsrc = s_src[warp];
-    // the stored stream as words (fewer than 2^32: slots are 32-bit), zero
-    // outside it; its last bytes make a word of their own
+    // the stored stream as words, zero outside it; its last bytes make a word
+    // of their own.  The buffer may be larger than slots can name: 2^32 codes
+    // of 16 bits lie in the first 2^31 words, so more are not counted.
     const u32* const words = reinterpret_cast<const u32*>(a.codes);
-    const u32 n_words = (u32)(a.codes_bytes / 4);
+    const u64 all_words = a.codes_bytes / 4;
+    const u32 n_words = all_words < (1ull << 31) ? (u32)all_words : 1u << 31;
     u32 tail = 0;
-    for (u32 q = 0; q < (u32)(a.codes_bytes & 3u); ++q) tail |= (u32)__ldg(a.codes + 4ull * n_words + q) << (8 * q);
+    for (u32 q = 0; q < (u32)(a.codes_bytes & 3u); ++q) tail |= (u32)__ldg(a.codes + 4 * all_words + q) << (8 * q);
     auto word = [&](u32 i) { return i < n_words ? __ldg(words + i) : (i == n_words ? tail : 0u); };
     for (u32 c = blockIdx.x * (kRowBlock / 32) + warp; c < n_chunks; c += gridDim.x * (kRowBlock / 32)) {
         const u32 k0 = row_of[c];
