@@ -39,7 +39,11 @@ __device__ __forceinline__ void cluster_arrive() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// (.aligned: the warp's lanes meet first, whatever branches they come from)
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 // A word of the same shared variable in block `rank` of the cluster.
 __device__ __forceinline__ u64 ld_cluster(const u64* a, u32 rank) {
     u32 addr;
