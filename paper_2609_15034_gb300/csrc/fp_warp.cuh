@@ -42,14 +42,6 @@ __device__ __forceinline__ Elem wt_unpack(u64 w) {
     return Elem{w & 0xffffffull, (w >> 24) & 0xffffffull, (u32)((w >> 48) & 3u)};
 }
 
-// A read-only load that stays where it is written (the compiler may move
-// __ldg() down to its use, behind the work that should hide it).
-__device__ __forceinline__ u32 ld_here(const u32* a) {
-    u32 v;
-    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(a));
-    return v;
-}
-
 // A lane's run of tokens appended to the warp's staging area as aligned
 // 64-bit words: `m` bytes of the current word (at `at`) are in c0, c1.
 //
@@ -782,14 +774,17 @@ struct WarpCore {
         u32 first, left;   // the lane's first boundary, boundaries from it to the tile's end
         u32 pos[PB];
     };
-    // Boundaries [lo, hi), clamped to the column's; issues the loads.
+    // Boundaries [lo, hi), clamped to the column's; issues the loads (in
+    // order: they stay ahead of the assembly that hides them, and off the
+    // read-only path, since the one-cluster decode may have started before
+    // the kernel that writes the column ended).
     static __device__ __forceinline__ void strings_begin(const DecodeParams& p, u32 lo, u32 hi, Strings& sb) {
         const u32 nb_col = p.n_strings + 1u;
         hi = min(hi, nb_col);
         sb.first = min(lo, nb_col) + (threadIdx.x & 31u);
         sb.left = sb.first < hi ? hi - sb.first : 0u;
 #pragma unroll
-        for (int j = 0; j < PB; ++j) sb.pos[j] = 32u * j < sb.left ? ld_here(p.code_offsets + sb.first + 32u * j) : 0u;
+        for (int j = 0; j < PB; ++j) sb.pos[j] = 32u * j < sb.left ? in_order(p.code_offsets + sb.first + 32u * j) : 0u;
     }
 
     // Assemble warp tile t of column (p, x) from its codes and token lengths
@@ -956,7 +951,7 @@ struct WarpCore {
             first += 32u * PB;
             left -= 32u * PB;
 #pragma unroll
-            for (int j = 0; j < PB; ++j) sb.pos[j] = 32u * j < left ? ld_here(p.code_offsets + first + 32u * j) : 0u;
+            for (int j = 0; j < PB; ++j) sb.pos[j] = 32u * j < left ? in_order(p.code_offsets + first + 32u * j) : 0u;
         }
         __syncwarp();   // the areas are reused by the next tile
         return tile_incl | ((u64)tile_out_state << 63);
