@@ -363,6 +363,7 @@ fp_status run_rows(fp_codec codec, const fp_dict* dict, const void* d_codes, uin
     p.codes_bytes = RL.codes_bytes;
     p.max_slots = dec_slots;
     p.code_offsets = reinterpret_cast<const uint32_t*>(rows + RL.o_v);
+    p.own_column = 1;
     p.n_strings = n_rows;
     p.out = d_out_bytes;
     p.capacity = size_only ? 0 : out_capacity;

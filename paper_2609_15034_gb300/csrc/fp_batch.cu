@@ -812,6 +812,8 @@ cudaError_t launch_kernels(const BatchKernel& BK, const BatchParams& bp, const I
     // Staged: a reduce per codec and the index pass, the scan, a decode per
     // codec.  Inside each of the two groups a launch may start in the tail of
     // the one before it (they share nothing; each ends only after that one).
+    // A group's first launch is an ordinary one: all that the group reads was
+    // complete before it began, so the others read it without a wait.
     auto launch = [&](const void* k, uint32_t blocks, int threads, size_t smem, void** a, bool early) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(blocks);

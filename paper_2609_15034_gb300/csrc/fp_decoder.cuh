@@ -86,6 +86,15 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 // launch of a call) is read after grid_wait() through after_wait() pointers
 // or in_order() loads, never with __ldg(): the read-only path may be read
 // ahead of the wait.
+//
+// The launches after a call's first read the caller's column (code offsets, a
+// warp's first codes) ahead of their own wait.  Its writers have ended by
+// then: the first launch waits for them and only afterwards lets the next one
+// start, which in turn lets the one after it start, so every write of theirs is
+// in L2 before a block of those launches begins.  An earlier launch may have
+// left older lines in L1, so these reads go past it (in_order_l2(), __ldcg(),
+// bulk copies).  Launches that read a column made by the call itself
+// (own_column) wait before they read any of it.
 template <class T>
 __device__ __forceinline__ const T* after_wait(const T* a) {
     const T* r;
@@ -509,18 +518,21 @@ __device__ void combine_and_store(uint4* chunk, uint4 acc, u32 lo, u32 hi, int m
 
 // The column's slot range [c_begin, c_end) from code_offsets[0] and
 // code_offsets[n], clamped to the code buffer (x.bad when it had to be).
+// AHEAD: read before the kernel's wait (past L1).
+template <bool AHEAD = false>
 __device__ __forceinline__ void slot_range(const DecodeParams& p, Extent& x) {
-    x.c_begin = in_order(p.code_offsets);
-    x.c_end = in_order(p.code_offsets + p.n_strings);
+    x.c_begin = AHEAD ? in_order_l2(p.code_offsets) : in_order(p.code_offsets);
+    x.c_end = AHEAD ? in_order_l2(p.code_offsets + p.n_strings) : in_order(p.code_offsets + p.n_strings);
     x.bad = 0u;
     if (x.c_end > p.max_slots) { x.c_end = p.max_slots; x.bad = 1u; }
     if (x.c_begin > x.c_end) { x.c_begin = x.c_end; x.bad = 1u; }
 }
 
 // Single-column tiling: the tiles that cover [c_begin, c_end).
+template <bool AHEAD = false>
 __device__ __forceinline__ Extent column_extent(const DecodeParams& p, u64 tile) {
     Extent x;
-    slot_range(p, x);
+    slot_range<AHEAD>(p, x);
     x.first_tile = x.c_begin / tile;
     const u64 end_tile = (x.c_end + tile - 1) / tile;
     x.n_tiles = end_tile > x.first_tile ? end_tile - x.first_tile : 1;

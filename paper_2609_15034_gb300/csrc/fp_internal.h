@@ -73,7 +73,7 @@ struct DecodeParams {
     unsigned long long* total_out;    // where this column's decoded size goes
     const uint32_t* first;            // tile -> first string boundary it owns (index pass)
     uint32_t packed_bits;             // cascaded codes: bits per code (packed decode only; else 0)
-    uint32_t pad_;
+    uint32_t own_column;              // 1: the call's own launches make the column (selective decode)
 };
 
 // Tiles of a column: a tile is `tile` consecutive code slots, tile u covers

@@ -199,13 +199,15 @@ struct WarpCore {
     }
 
     // Raw code words of the lane (LANE_WORDS words); false if they run past
-    // the buffer (then load_guarded() is used).
+    // the buffer (then load_guarded() is used).  AHEAD: read before the
+    // kernel's wait (past L1).
+    template <bool AHEAD = false>
     static __device__ __forceinline__ bool load_fast(const DecodeParams& p, u64 q0, u32 (&wv)[LANE_WORDS]) {
         if (PACKED) {
             const u64 w0 = (q0 * p.packed_bits) >> 5;   // the word holding the lane's first bit
             const u32 n = packed_words(p.packed_bits);
             if ((w0 + n) * 4 > p.codes_bytes) return false;
-            load_packed(reinterpret_cast<const u32*>(p.codes) + w0, n, wv);
+            load_packed<AHEAD>(reinterpret_cast<const u32*>(p.codes) + w0, n, wv);
             return true;
         }
         const u64 b0 = q0 * WBITS / 8;   // q0 is a multiple of K, K a multiple of 8
@@ -214,14 +216,14 @@ struct WarpCore {
             const uint4* src = reinterpret_cast<const uint4*>(p.codes + b0);
 #pragma unroll
             for (int v = 0; v < LANE_BYTES / 16; ++v) {
-                const uint4 a = __ldcs(src + v);
+                const uint4 a = AHEAD ? __ldcg(src + v) : __ldcs(src + v);
                 wv[4 * v] = a.x; wv[4 * v + 1] = a.y; wv[4 * v + 2] = a.z; wv[4 * v + 3] = a.w;
             }
         } else {
             const uint2* src = reinterpret_cast<const uint2*>(p.codes + b0);
 #pragma unroll
             for (int v = 0; v < LANE_BYTES / 8; ++v) {
-                const uint2 a = __ldcs(src + v);
+                const uint2 a = AHEAD ? __ldcg(src + v) : __ldcs(src + v);
                 wv[2 * v] = a.x; wv[2 * v + 1] = a.y;
             }
         }
@@ -313,9 +315,10 @@ struct WarpCore {
     // from a multiple of 16 bits on, so they begin at a word, or (odd b, odd
     // lanes) in the middle of one, and lie in these words either way.
     static __device__ __forceinline__ u32 packed_words(u32 b) { return K == 32 ? b : (b + 1u) >> 1; }
+    template <bool AHEAD = false>
     static __device__ __forceinline__ void load_packed(const u32* src, u32 n, u32* wv) {
 #pragma unroll
-        for (int i = 0; i < LANE_WORDS; ++i) wv[i] = (u32)i < n ? __ldcs(src + i) : 0u;
+        for (int i = 0; i < LANE_WORDS; ++i) wv[i] = (u32)i < n ? (AHEAD ? __ldcg(src + i) : __ldcs(src + i)) : 0u;
     }
     // `o`: the bit the codes begin at in wv[0], 0 or 16.
     template <int B>
@@ -738,8 +741,9 @@ struct WarpCore {
     static constexpr int PB = K / 8;
 
     // Issue the loads of tile t (every lane of the warp, the tile before it
-    // read from area.codes): its codes, which are the caller's input, and
-    // what the passes before the decode made.
+    // read from area.codes): its codes, and what the passes before the decode
+    // made.  AHEAD: the codes before the kernel's wait (past L1).
+    template <bool AHEAD = false>
     static __device__ __forceinline__ void fetch_codes(const DecodeParams& p, const Extent& x, u64 t, Area& area,
                                                        const CodeBar& cb, Fetch& f) {
         if constexpr (BULK_CODES) {
@@ -752,7 +756,7 @@ struct WarpCore {
                 mbar_arrive(cb.bar);
             }
         } else {
-            f.in = load_fast(p, lane_q0(x, t), f.wv);
+            f.in = load_fast<AHEAD>(p, lane_q0(x, t), f.wv);
         }
     }
     // The launches (or phases) before this one wrote these while it was
@@ -1011,7 +1015,7 @@ struct WarpCore {
         CodeBar cb;
         cb.init(bar);
         Fetch cur;
-        fetch_codes(p, x, t, area, cb, cur);
+        fetch_codes<true>(p, x, t, area, cb, cur);
         grid_wait();   // the launch before (none before a cooperative launch's phases)
         fetch_scanned(ex, p.first, t, cur);
         for (; t < x.n_tiles; t += step) {
@@ -1367,18 +1371,21 @@ __device__ __forceinline__ void renew_launch(WsHeader* ws) {
     ws->epoch = ne ? ne : 1u;
 }
 
-// Everything that does not depend on the reduce (the first ticket, the launch
-// tag, the column's extent) is fetched while the reduce still runs: on a
-// small column the scan is a chain of global round trips.
+// Everything that does not depend on the reduce (the first ticket and the
+// launch tag, which the call before left, the caller's extent) is fetched,
+// past L1, while the reduce still runs: on a small column the scan is a chain
+// of global round trips (FSST-8, 30k strings, with all of it and the decode's
+// first codes after the wait: 13.2 us a call against 12.3).
 template <bool FSST>
 __global__ void __launch_bounds__(256, 4) tiles_scan_kernel(const DecodeParams p, u32 tile, const u64* agg, u64* ex,
                                                             unsigned long long* status) {
     __shared__ ScanShared sh;
     WsHeader* ws = p.ws;
     grid_release();   // the decode may start launching (its blocks stage the dictionary, then wait)
+    if (p.own_column) grid_wait();
     if (threadIdx.x == 0) sh.ticket = atomicAdd(&ws->tile_counter, 1u);
     const u32 epoch = *(volatile u32*)&ws->epoch;
-    const u64 n = column_extent(p, tile).n_tiles;
+    const u64 n = column_extent<true>(p, tile).n_tiles;
     const u64 n_blocks = (n + kScanTile - 1) / kScanTile;
     grid_wait();      // the reduce's elements
     for (;;) {
@@ -1412,7 +1419,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) warp_decode_kernel(const Decode
         C::stage_dict(p, s_dict, s_lens, NW * 32);
         __syncthreads();
     }
-    const Extent x = column_extent(p, C::TILE);
+    if (p.own_column) grid_wait();
+    const Extent x = column_extent<true>(p, C::TILE);
     const uint8_t* lens = LSMEM ? s_lens : p.dict.lens;
     u32 err = 0;
     // decode_tiles() fetches the first tile's codes, then waits for the tile
