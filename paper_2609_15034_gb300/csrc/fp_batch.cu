@@ -214,6 +214,7 @@ __device__ __forceinline__ void decode_queue(const BatchParams& bp, int q, u64 t
         rn = r2;
     }
     phase = cb.phase;
+    cb.drain(bp.ws);
     // the area and the record slot are reused by the next queue, whose bulk
     // copies may land where this one stored
     C::stage_free(lane);
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) wbatch_decode_kernel(const Batc
     __shared__ __align__(8) u64 s_code_bar[NW];
     u64* bar = s_code_bar + warp;
     if ((threadIdx.x & 31u) == 0u) {
-        mbar_init(bar, 1u);
+        mbar_init(bar, FP_COPY_ARRIVALS);
         mbar_init_fence();
     }
     __syncwarp();
@@ -305,13 +306,13 @@ __global__ void __launch_bounds__(kUnitWarps * 32, 1) unit_decode_kernel(const B
         return u < n_units ? __ldg(bp.units[q] + u) : make_uint4(0u, 0u, 0u, 0u);
     };
     if (threadIdx.x == 0) {
-        mbar_init(&s_bar, 1u);
+        mbar_init(&s_bar, FP_COPY_ARRIVALS);
         mbar_init_fence();
         s_unit[0] = take();
     }
     __syncthreads();
     const void* staged = nullptr;   // the table in shared memory
-    u32 bar_phase = 0u;
+    u32 bar_phase = 0u, late = 0u;   // late: a wait for tables gave up, no more copies of them
     for (u32 i = 0;; ++i) {
         const uint4 unit = s_unit[i & 1u];
         if (unit.z == 0u) break;
@@ -323,10 +324,10 @@ __global__ void __launch_bounds__(kUnitWarps * 32, 1) unit_decode_kernel(const B
         if (p.dict.table != staged) {
             const bool aligned =
                 ((reinterpret_cast<uintptr_t>(p.dict.table) | reinterpret_cast<uintptr_t>(p.dict.lens)) & 15u) == 0u;
-            if (C::BULK_STAGE && aligned) {
+            if (C::BULK_STAGE && aligned && !late) {
                 if (threadIdx.x == 0) C::bulk_tables(p, s_dict, s_lens, &s_bar);
-                mbar_wait(&s_bar, bar_phase, p.ws);
-                bar_phase ^= 1u;
+                late = C::wait_tables(p, s_dict, s_lens, &s_bar, bar_phase, kUnitWarps * 32);
+                if (!late) bar_phase ^= 1u;
             } else {
                 C::stage_dict(p, s_dict, s_lens, kUnitWarps * 32);
                 __syncthreads();
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(kUnitWarps * 32, 1) unit_decode_kernel(const B
             staged = p.dict.table;
         }
         const u64* ex = bp.ex + rec.wt_base;
-        u32 err = 0;
+        u32 err = late;
         u64 t = unit.y + warp;
         const u64 t_end = (u64)unit.y + unit.z;
         if (t < t_end) {
@@ -352,6 +353,7 @@ __global__ void __launch_bounds__(kUnitWarps * 32, 1) unit_decode_kernel(const B
         __syncthreads();   // the tables and the record are replaced
     }
     C::stage_free(lane);
+    cb.drain(bp.ws);
     grid_wait();
 }
 

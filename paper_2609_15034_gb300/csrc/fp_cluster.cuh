@@ -68,8 +68,9 @@ __global__ void __launch_bounds__(NW * 32, 1) cluster_decode_kernel(const Decode
     typename C::Area& area = reinterpret_cast<typename C::Area*>(smem_raw + C::STAGED_BYTES)[threadIdx.x >> 5];
     const u32 lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const u32 rank = cluster_rank(), blocks = cluster_size();
+    u32 err = 0;
     if (C::BULK_STAGE) {
-        C::stage_dict_bulk(pp, s_dict, s_lens, &s_bar, NW * 32);
+        err = C::stage_dict_bulk(pp, s_dict, s_lens, &s_bar, NW * 32);
     } else if (DSMEM) {
         C::stage_dict(pp, s_dict, s_lens, NW * 32);
         __syncthreads();
@@ -84,7 +85,6 @@ __global__ void __launch_bounds__(NW * 32, 1) cluster_decode_kernel(const Decode
     // the block's tiles [b0, b1), the warp's [t0, t1)
     const u32 b0 = (u32)((u64)n * rank / blocks), b1 = (u32)((u64)n * (rank + 1) / blocks);
     const u32 t0 = b0 + (u32)((u64)(b1 - b0) * warp / NW), t1 = b0 + (u32)((u64)(b1 - b0) * (warp + 1) / NW);
-    u32 err = 0;
     u32 wv[C::LANE_WORDS];
     bool in = false;
     if (t0 < t1) in = C::load_fast(p, C::lane_q0(x, t1 - 1), wv);

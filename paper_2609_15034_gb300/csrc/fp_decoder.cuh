@@ -659,7 +659,15 @@ __device__ __forceinline__ void async_fence() { asm volatile("fence.proxy.async.
 // the pipeline still runs to its end (with wrong positions, every write in
 // bounds), so the workers, the scan warp and the producer keep seeing the
 // same ring state and every named barrier stays matched.
-constexpr u64 kWaitLimitNs = 4000000000ull;
+#ifndef FP_WAIT_LIMIT_NS
+#define FP_WAIT_LIMIT_NS 4000000000ull
+#endif
+constexpr u64 kWaitLimitNs = FP_WAIT_LIMIT_NS;
+// Arrivals that the barrier of the warp-tile decoder's copies waits for (a
+// test builds it with one more than are ever made: every wait runs out).
+#ifndef FP_COPY_ARRIVALS
+#define FP_COPY_ARRIVALS 1u
+#endif
 
 // Wait for a phase of `bar`; gives up (status ERRB_TIMEOUT, abort flag) after
 // kWaitLimitNs.  Returns false on giving up.

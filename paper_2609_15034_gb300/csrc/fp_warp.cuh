@@ -649,26 +649,35 @@ struct WarpCore {
     // The same staging by the bulk-copy engine where the staged layout is the
     // stored one (no planes, no literals): thread 0 issues the two
     // copies (cp.async.bulk, completion counted on one mbarrier) and every
-    // thread waits for them, bounded (a wait that gives up sets
-    // ERRB_TIMEOUT).  Falls back to the loads above for tables that are not
-    // 16-byte aligned.  Every thread of the block calls it; returns synchronised.
+    // thread waits for them, bounded.  Falls back to the loads above for tables
+    // that are not 16-byte aligned, and where a wait gave up (after one more
+    // for the copies in flight): then the result is ERRB_TIMEOUT, else 0.
+    // Every thread of the block calls it; returns synchronised.
     static constexpr bool BULK_STAGE = LSMEM && !LITTAB && (!DSMEM || TOK8 || W == 16);
-    static __device__ __forceinline__ void stage_dict_bulk(const DecodeParams& p, uint4* s_dict, uint8_t* s_lens,
-                                                           u64* bar, int nthreads) {
+    static __device__ __forceinline__ u32 stage_dict_bulk(const DecodeParams& p, uint4* s_dict, uint8_t* s_lens,
+                                                          u64* bar, int nthreads) {
         const bool aligned =
             ((reinterpret_cast<uintptr_t>(p.dict.table) | reinterpret_cast<uintptr_t>(p.dict.lens)) & 15u) == 0u;
         if (!aligned) {
             stage_dict(p, s_dict, s_lens, nthreads);
             __syncthreads();
-            return;
+            return 0u;
         }
         if (threadIdx.x == 0) {
-            mbar_init(bar, 1u);
+            mbar_init(bar, FP_COPY_ARRIVALS);
             mbar_init_fence();
             bulk_tables(p, s_dict, s_lens, bar);
         }
         __syncthreads();   // the barrier is initialised before anyone waits on it
-        mbar_wait(bar, 0u, p.ws);
+        return wait_tables(p, s_dict, s_lens, bar, 0u, nthreads);
+    }
+    static __device__ __forceinline__ u32 wait_tables(const DecodeParams& p, uint4* s_dict, uint8_t* s_lens, u64* bar,
+                                                      u32 phase, int nthreads) {
+        if (!__syncthreads_or(!mbar_wait(bar, phase, p.ws))) return 0u;
+        mbar_wait(bar, phase, p.ws);
+        stage_dict(p, s_dict, s_lens, nthreads);
+        __syncthreads();
+        return ERRB_TIMEOUT;
     }
     // Issue the two copies (one thread; `bar` is initialised).
     static __device__ __forceinline__ void bulk_tables(const DecodeParams& p, uint4* s_dict, uint8_t* s_lens, u64* bar) {
@@ -722,16 +731,29 @@ struct WarpCore {
         u64 ex;
         u32 lo, hi;
     };
-    // The warp's mbarrier for those copies and the phase of the next one.
+    // The warp's mbarrier for those copies and the phase of the next one; 2
+    // more once a wait has given up, after which the warp issues no copies.
     struct CodeBar {
         u64* bar;
         u32 phase;
+        __device__ __forceinline__ bool usable() const { return phase < 2u; }
+        // The copy has landed (every lane of the warp; false: none waits for it any more).
+        __device__ __forceinline__ bool wait(WsHeader* ws) {
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, phase, ws));
+            phase = ok ? phase ^ 1u : phase | 2u;
+            return ok;
+        }
+        // Before the area is used for something else, or the block ends: once
+        // more for a copy that was given up.
+        __device__ __forceinline__ void drain(WsHeader* ws) const {
+            if (!usable()) mbar_wait(bar, phase & 1u, ws);
+        }
         // Every lane of the warp calls it, before the first fetch().
         __device__ __forceinline__ void init(u64* b) {
             bar = b;
             phase = 0u;
             if ((threadIdx.x & 31u) == 0u) {
-                mbar_init(bar, 1u);
+                mbar_init(bar, FP_COPY_ARRIVALS);
                 mbar_init_fence();
             }
             __syncwarp();
@@ -749,7 +771,7 @@ struct WarpCore {
         if constexpr (BULK_CODES) {
             const u32 tb = tile_bytes(p);
             const u64 b0 = (x.first_tile + t) * tb;   // a multiple of 16, as tb is
-            f.in = b0 + tb <= p.codes_bytes;
+            f.in = b0 + tb <= p.codes_bytes && cb.usable();
             if (f.in && (threadIdx.x & 31u) == 0u) {
                 mbar_expect_tx(cb.bar, tb);
                 bulk_g2s(area.codes, p.codes + b0, tb, cb.bar);
@@ -985,11 +1007,11 @@ struct WarpCore {
         R r;
         if constexpr (BULK_CODES) {
             u32 wv[LANE_WORDS];
-            const bool in = f.in;
+            bool in = f.in;
             if (in) {
-                mbar_wait(cb.bar, cb.phase, p.ws);
-                cb.phase ^= 1u;
-                load_staged(p, area.codes, lane, wv);
+                in = cb.wait(p.ws);
+                if (in) load_staged(p, area.codes, lane, wv);
+                else err |= ERRB_TIMEOUT;   // the tile's codes by guarded loads
             }
             __syncwarp();   // the codes have left the area
             next();
@@ -1028,6 +1050,7 @@ struct WarpCore {
             cur = nxt;
         }
         stage_free(threadIdx.x & 31u);   // shared memory outlives the copies from it
+        cb.drain(p.ws);                  // and the copies to it
     }
 };
 
@@ -1413,8 +1436,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) warp_decode_kernel(const Decode
     typename C::Area* areas = reinterpret_cast<typename C::Area*>(smem_raw + C::STAGED_BYTES);
     __shared__ __align__(8) u64 s_bar;
     __shared__ __align__(8) u64 s_code_bar[NW];
+    u32 err = 0;
     if (C::BULK_STAGE) {
-        C::stage_dict_bulk(p, s_dict, s_lens, &s_bar, NW * 32);
+        err = C::stage_dict_bulk(p, s_dict, s_lens, &s_bar, NW * 32);
     } else if (LSMEM) {
         C::stage_dict(p, s_dict, s_lens, NW * 32);
         __syncthreads();
@@ -1422,7 +1446,6 @@ __global__ void __launch_bounds__(NW * 32, MINB) warp_decode_kernel(const Decode
     if (p.own_column) grid_wait();
     const Extent x = column_extent<true>(p, C::TILE);
     const uint8_t* lens = LSMEM ? s_lens : p.dict.lens;
-    u32 err = 0;
     // decode_tiles() fetches the first tile's codes, then waits for the tile
     // scan's offsets: staging and fetch overlap the scan
     C::decode_tiles(p, x, ex, (u64)blockIdx.x * NW + (threadIdx.x >> 5), (u64)gridDim.x * NW, s_dict, lens,
