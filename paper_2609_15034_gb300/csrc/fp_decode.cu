@@ -237,7 +237,17 @@ cudaError_t launch_decode(int codec, const Variant& var, const DecodeParams& p_i
     const int nw = var.threads / 32;
     uint64_t dg = (n_wt_max + nw - 1) / nw;
     if (dg > (uint64_t)grid) dg = (uint64_t)grid;
-    return launch_after(var.kernel, dim3((unsigned)dg), dim3(var.threads), dargs, var.smem_bytes, stream);
+    e = launch_after(var.kernel, dim3((unsigned)dg), dim3(var.threads), dargs, var.smem_bytes, stream);
+    if (e != cudaSuccess) {
+        // the scan is enqueued and the decode, which renews the launch state
+        // (renew_launch()), is not: the tickets go back to zero, the stall
+        // settings too, and no look-back word keeps this launch's tag
+        char* ws = reinterpret_cast<char*>(p.ws);
+        cudaMemsetAsync(ws + kWsCounters, 0, kWsCounterBytes, stream);
+        cudaMemsetAsync(ws + offsetof(WsHeader, spin_limit), 0, 2 * sizeof(unsigned), stream);
+        cudaMemsetAsync(base + L.o_status, 0, L.o_extent - L.o_status, stream);
+    }
+    return e;
 }
 
 }  // namespace fp

@@ -1,6 +1,7 @@
 // Internal declarations shared by the library's host and device sources.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <vector>
 #include <cuda_runtime.h>
@@ -24,21 +25,25 @@ constexpr uint32_t ERRB_MISMATCH = 16u;
 // status words of the single-pass prefix scan (one u64 per tile, at
 // `kWsHeaderBytes`) and by the tile -> first string index (tiles + 1 u32).
 struct WsHeader {
-    unsigned int tile_counter;   // next tile ticket
-    unsigned int exit_counter;   // blocks that have finished
     unsigned int epoch;          // launch generation tag of tile status words
-    unsigned int status;         // sticky ERRB_* bits
-    unsigned long long rows_slots;   // selective decode: code slots of the selected rows
-    unsigned long long total;    // decoded size of the last launch
-    unsigned int abort;          // set when a bounded wait gave up
-    unsigned int queue_counter[3];   // batched decode: next tile ticket of each codec queue
     unsigned int spin_limit;     // polls before a look-back gives up (0 = the built-in limit); reset per launch
     unsigned int bar_count;      // one-launch decode: blocks arrived at the current grid barrier
     unsigned int bar_gen;        // one-launch decode: grid barriers passed
+    unsigned long long rows_slots;   // selective decode: code slots of the selected rows
+    unsigned long long total;    // decoded size of the last launch
+    // zero when a call's launches begin; the launches leave them so
+    unsigned int tile_counter;   // next tile ticket
+    unsigned int exit_counter;   // blocks that have finished
+    unsigned int abort;          // set when a bounded wait gave up
+    unsigned int queue_counter[3];   // batched decode: next tile ticket of each codec queue
     unsigned int unit_counter[4];    // staged batch: next unit of each codec, decode
     unsigned int reduce_counter[4];  // and reduce
+    unsigned int status;         // sticky ERRB_* bits
     unsigned int pad[9];
 };
+// The counters alone, and with the status word behind them.
+constexpr size_t kWsCounters = offsetof(WsHeader, tile_counter);
+constexpr size_t kWsCounterBytes = offsetof(WsHeader, status) - kWsCounters;
 constexpr size_t kWsHeaderBytes = 128;
 static_assert(sizeof(WsHeader) == kWsHeaderBytes, "workspace header size");
 
