@@ -1165,8 +1165,9 @@ fp_status wave_launch(WaveBuffers& W, const fp_chunk* chunks, uint32_t n, int co
     // earlier wave's table bytes can pass for a published word
     if (e == cudaSuccess) e = cudaMemsetAsync(base + L.o_ts, 0, L.status_words * sizeof(unsigned long long), stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(W.d_status, 0, n * sizeof(uint32_t), stream);
+    // the status, and the tickets that a wave drew whose launches were not all enqueued
     if (e == cudaSuccess)
-        e = cudaMemsetAsync(static_cast<char*>(W.d_hdr) + offsetof(WsHeader, status), 0, sizeof(unsigned), stream);
+        e = cudaMemsetAsync(static_cast<char*>(W.d_hdr) + kWsCounters, 0, kWsCounterBytes + sizeof(unsigned), stream);
     if (e != cudaSuccess) return cuda_fail(e, "wave upload");
     uint32_t split[2];
     int grid = 0;

@@ -301,9 +301,12 @@ void lane_launch(fp_server* S, Lane& L) {
     cudaError_t e = cudaSuccess;
     if (stt == FP_OK) e = cudaEventRecord(L.ev, L.s);
     if (stt != FP_OK || e != cudaSuccess) {
-        // the launch failed on the host: fail the wave's requests
+        // the launch failed on the host: fail the wave's requests, once the
+        // launches that were made are done with their buffers
+        const std::string why = stt != FP_OK ? fp_last_error() : cudaGetErrorString(e);
+        cudaStreamSynchronize(L.s);
         std::lock_guard<std::mutex> lk(S->mu);
-        S->sched_error = fp_last_error();
+        S->sched_error = why;
         for (Req* q : L.reqs) {
             q->status = stt != FP_OK ? (uint32_t)stt : (uint32_t)FP_ERR_CUDA;
             q->t_done = now_ns();

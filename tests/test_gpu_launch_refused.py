@@ -57,6 +57,42 @@ for first in range(3):
 print("passed")
 """
 
+SERVED = r"""
+import ctypes, sys
+import numpy as np
+import synth
+from test_gpu_serve import Page, collect, fetch, register
+import paper_2609_15034_gb300 as fp
+
+refuse = ctypes.CDLL(None).shim_refuse
+k = int(sys.argv[1])
+codecs = (synth.ONPAIR16, synth.ONPAIR12, synth.FSST8, synth.FSST12)
+pages = [Page(synth.column(c, 800 + 10 * c + s, n), key=10 * c + s) for c in codecs for s, n in ((1, 9000), (2, 7000))]
+srv = fp.Server(hbm_budget=256 << 20, n_streams=1, max_wave=1, batch_config=5)   # the staged launches
+register(srv, pages)
+
+
+def one(p):
+    p.submit(srv, tag=0)
+    (t, r), = collect(fp, srv, 1).items()
+    if r["status"] == fp.OK:
+        data, offs = fetch(fp, r)
+        assert np.array_equal(data, p.ref.data)
+        np.testing.assert_array_equal(offs, p.ref.offsets)
+    srv.release(t)
+    return r["status"]
+
+
+for a, b in zip(pages[::2], pages[1::2]):
+    assert one(a) == fp.OK
+    refuse(k)
+    assert one(b) == fp.ERR_CUDA
+    for p in (a, b, a):
+        assert one(p) == fp.OK
+srv.destroy()
+print("passed")
+"""
+
 
 def run(tmp_path, script, *args):
     c, so = tmp_path / "shim.c", tmp_path / "shim.so"
@@ -80,3 +116,9 @@ def gpu():
 @pytest.mark.parametrize("launch", [1, 2, 3])
 def test_decode_launch_refused(tmp_path, codec, launch):
     run(tmp_path, COLUMN, codec, launch)
+
+
+# of a wave of one chunk: reduce, index pass, decode (the scan is launched another way)
+@pytest.mark.parametrize("launch", [1, 2, 3])
+def test_wave_launch_refused(tmp_path, launch):
+    run(tmp_path, SERVED, launch)
