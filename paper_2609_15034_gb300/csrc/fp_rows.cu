@@ -168,19 +168,33 @@ __device__ __forceinline__ u32 bits_below(int b) { return b <= 0 ? 0u : (b >= 32
 
 // Pass 3: gather.  A warp writes a chunk of 32 groups of G virtual slots of
 // the compacted stream, a lane one group as whole words: 8 slots of 16 or 12
-// bits (4 or 3 words), 16 slots of 8 bits (4 words).  The rows of the chunk
-// (about 14 of 18 codes) are looked up in a window in shared memory, and a
-// row's part of a group is one window of aligned words of the stored stream
-// shifted into place: 5 or 4 word loads, where a byte or two per slot took up
-// to 16 loads and a search over all rows 20 more (1M rows of 18 12-bit codes:
-// GATHER_US).  Slots past the selected total (or the bound) are written as
-// zero and never decoded.
+// bits (4 or 3 words), 16 slots of 8 bits (4 words).  The chunk's rows (about
+// 14 of 18 codes, as many as slots of one code) pass through a window in
+// shared memory, and a row's part of a group is one window of aligned words of
+// the stored stream shifted into place, where a byte or two per slot took up
+// to 16 loads and a search over all rows 20 more.
+//
+// The window holds a chunk of one-code rows, so that every lane finds its rows
+// in the first one; with one of 64 rows the lanes past it searched global
+// memory row by row.  500k of 5M rows, a whole call, a byte or two per slot ->
+// window of 64 -> this: OnPair-12, 1 code a row 61.6 -> 73.9 -> 48.1 us, 2 codes
+// 58.0 -> 59.5 -> 37.9, 18 codes 122.9 -> 88.7 -> 90.2; FSST-8 64.3 -> 121.6 ->
+// 57.0, 63.8 -> 85.5 -> 45.6, 141.8 -> 81.6 -> 82.7.  A chunk of more rows than
+// kRowWindows windows hold (almost all of them empty) has the rest searched in
+// global memory.  Slots past the selected total (or the bound) are not written
+// and never decoded.
+constexpr u32 kRowWindows = 8;
+// Blocks per SM: FSST-8's window of 512 rows takes 32 KiB a block; with six
+// blocks L1 is left too little (18 codes a row: 103.5 us against 82.7).
+__host__ __device__ constexpr int row_gather_blocks(int codec) { return codec == FP_FSST8 ? 5 : 6; }
+
 template <int CODEC>
-__global__ void __launch_bounds__(kRowBlock) rows_gather_kernel(const RowsArgs a, const u32* v, const u32* src,
+__global__ void __launch_bounds__(kRowBlock, row_gather_blocks(CODEC)) rows_gather_kernel(const RowsArgs a, const u32* v, const u32* src,
                                                               const u32* row_of, uint8_t* out, u64 bound,
                                                               const WsHeader* ws) {
     constexpr int BITS = CODEC == FP_ONPAIR16 ? 16 : (CODEC == FP_FSST8 ? 8 : 12);
-    constexpr int G = CODEC == FP_FSST8 ? 16 : 8, CH = 32 * G, NW = G * BITS / 32, WIN = 64;
+    constexpr int G = CODEC == FP_FSST8 ? 16 : 8, CH = 32 * G, NW = G * BITS / 32;
+    constexpr u32 WIN = CODEC == FP_FSST8 ? 512 : 256;
     __shared__ u32 s_v[kRowBlock / 32][WIN + 1], s_src[kRowBlock / 32][WIN];
     grid_wait();
     grid_release();
@@ -202,59 +216,69 @@ __global__ void __launch_bounds__(kRowBlock) rows_gather_kernel(const RowsArgs a
     for (u32 q = 0; q < (u32)(a.codes_bytes & 3u); ++q) tail |= (u32)__ldg(a.codes + 4 * all_words + q) << (8 * q);
     auto word = [&](u32 i) { return i < n_words ? __ldg(words + i) : (i == n_words ? tail : 0u); };
     for (u32 c = blockIdx.x * (kRowBlock / 32) + warp; c < n_chunks; c += gridDim.x * (kRowBlock / 32)) {
-        const u32 k0 = row_of[c];
-        for (u32 i = lane; i <= (u32)WIN; i += 32u) {
-            wv[i] = v[min(k0 + i, m)];
-            if (i < (u32)WIN) wsrc[i] = k0 + i < m ? src[k0 + i] : 0u;
-        }
-        __syncwarp();
+        // the chunk's rows lie in [k0, k_end)
+        const u32 k0 = row_of[c], k_end = c + 1u < n_chunks ? row_of[c + 1u] + 1u : m;
         const u32 v0 = c * (u32)CH + lane * G;
         u32 acc[NW] = {};
         const u32 left = v0 < total ? min(total - v0, (u32)G) : 0u;
-        u32 j = 0, i = WIN;   // i: the row in the window
-        while (j < left) {
-            // the row of slot v0 + j (non-empty, so its id passed the
-            // checks): its first virtual slot, its end, its first stored slot
-            const u32 pos = v0 + j;
-            u32 vs, ve, sb;
-            if (pos < wv[WIN]) {
-                if (j == 0u) {
-                    i = 0u;
-#pragma unroll
-                    for (u32 d = WIN / 2; d > 0; d >>= 1)
-                        if (wv[i + d] <= pos) i += d;
-                } else {
-                    do ++i;
-                    while (wv[i + 1] <= pos);
-                }
-                vs = wv[i];
-                ve = wv[i + 1];
-                sb = wsrc[i];
-            } else {
-                u32 lo = k0, hi = m;   // v[lo] <= pos < v[hi]
-                while (hi - lo > 1u) {
-                    const u32 mid = lo + (hi - lo) / 2u;
-                    if (v[mid] <= pos) lo = mid;
-                    else hi = mid;
-                }
-                vs = v[lo];
-                ve = v[lo + 1];
-                sb = src[lo];
-            }
+        u32 j = 0;   // slots of the group done
+        // slots j .. of the group from the row of slot v0 + j (non-empty, so
+        // its id passed the checks): its first virtual slot, its end, its
+        // first stored slot
+        auto take = [&](u32 vs, u32 ve, u32 sb) {
+            const u32 end = min(left, ve - v0);
             // the words from the stored bit of the group's slot 0 on, as if
-            // the row began early enough and ended late enough: the rows
-            // after it overwrite the rest
+            // the row began early enough (only those that slots j .. end - 1
+            // touch are loaded: 2 of 5 for a row of one code)
             const long long bit = (long long)BITS * ((long long)sb + v0 - vs);
             const u32 w0 = (u32)(bit >> 5);
+            const u32 q_lo = j * BITS / 32u, q_hi = (end * BITS - 1u) / 32u + 1u;
             u32 x[NW + 1];
 #pragma unroll
-            for (int q = 0; q <= NW; ++q) x[q] = word(w0 + q);
+            for (int q = 0; q <= NW; ++q) x[q] = (u32)q >= q_lo && (u32)q <= q_hi ? word(w0 + q) : 0u;
 #pragma unroll
             for (int q = 0; q < NW; ++q) {
                 const u32 keep = j ? bits_below((int)j * BITS - 32 * q) : 0u;
                 acc[q] = (acc[q] & keep) | (__funnelshift_r(x[q], x[q + 1], (u32)bit) & ~keep);
             }
-            j = min(left, ve - v0);
+            j = end;
+        };
+        u32 base = k0;
+        for (u32 w = 0; w < kRowWindows; ++w) {
+            const u32 n_in = min(k_end - base, WIN);
+            for (u32 i = lane; i <= n_in; i += 32u) {
+                wv[i] = v[base + i];
+                if (i < n_in) wsrc[i] = src[base + i];
+            }
+            __syncwarp();
+            const u32 covered = wv[n_in], step = n_in > 1u ? 1u << (31 - __clz(n_in - 1u)) : 0u;
+            u32 i = n_in;   // the row in the window
+            while (j < left && v0 + j < covered) {
+                const u32 pos = v0 + j;
+                if (i == n_in) {
+                    i = 0u;
+                    for (u32 d = step; d > 0u; d >>= 1)
+                        if (i + d < n_in && wv[i + d] <= pos) i += d;
+                } else {
+                    do ++i;
+                    while (wv[i + 1] <= pos);
+                }
+                take(wv[i], wv[i + 1], wsrc[i]);
+            }
+            base += n_in;
+            const bool done = __all_sync(0xffffffffu, j >= left) || base >= k_end;
+            __syncwarp();   // the window is refilled
+            if (done) break;
+        }
+        while (j < left && base < k_end) {
+            const u32 pos = v0 + j;
+            u32 hi = k_end;   // v[base] <= pos < v[hi]
+            while (hi - base > 1u) {
+                const u32 mid = base + (hi - base) / 2u;
+                if (v[mid] <= pos) base = mid;
+                else hi = mid;
+            }
+            take(v[base], v[base + 1], src[base]);
         }
         if (left < (u32)G)
 #pragma unroll
@@ -270,7 +294,6 @@ __global__ void __launch_bounds__(kRowBlock) rows_gather_kernel(const RowsArgs a
                 w[2] = acc[2];
             }
         }
-        __syncwarp();   // the window is refilled
     }
 }
 
@@ -328,7 +351,8 @@ cudaError_t launch_rows_gather(int codec, const RowsArgs& a, uint64_t selected_s
     if (e != cudaSuccess || !gather) return e;
     const uint64_t per_block = (uint64_t)row_chunk(codec) * (kRowBlock / 32);
     uint64_t grid = (selected_slots + per_block - 1) / per_block;
-    if (grid > (uint64_t)sms * 8) grid = (uint64_t)sms * 8;
+    const uint64_t grid_max = (uint64_t)sms * row_gather_blocks(codec);
+    if (grid > grid_max) grid = grid_max;
     if (grid < 1) grid = 1;
     const u32 g = (u32)grid;
     switch (codec) {
