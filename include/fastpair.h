@@ -540,7 +540,9 @@ fp_status fp_serve_destroy(fp_server* server);
  * fp_variant_selected  the variant selected for the codec, or with none
  *                   selected the default for large code buffers.
  * fp_variant_for    the variant fp_decode uses for a code buffer of
- *                   codes_bytes bytes (-1 for an unknown codec).
+ *                   codes_bytes bytes (-1 for an unknown codec); with 2^17
+ *                   strings or more, a default shape of one cluster gives
+ *                   way to three launches.
  */
 int fp_variant_count(fp_codec codec);
 fp_status fp_variant_info(fp_codec codec, int v, uint32_t* threads, uint32_t* slots_per_thread,

@@ -3,6 +3,7 @@
 // and kernel launches.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdarg>
 #include <cstdio>
@@ -146,6 +147,15 @@ int selected_variant(int codec, uint64_t max_slots, int width) {
     return variant_default(codec, max_slots, width);
 }
 
+// The same for a column of n_strings strings: one of many strings for its
+// code slots takes the default just above the one-cluster decode's sizes.
+int column_variant(int codec, uint64_t max_slots, int width, uint32_t n_strings) {
+    const int v = selected_variant(codec, max_slots, width);
+    if (g_selected[codec].load() >= 0 || n_strings < cluster_strings_limit()) return v;
+    const Variant* var = variant_get(codec, v);
+    return var && var->warp_tiles == 3 ? variant_default(codec, std::max<uint64_t>(max_slots, 1ull << 17), width) : v;
+}
+
 struct DevInfo {
     int sms = 0;
     std::map<const void*, int> blocks_per_sm;
@@ -274,7 +284,7 @@ fp_status run_decode(fp_codec codec, const fp_dict* dict, const void* d_codes, u
     const uint64_t max_slots = packed_bits ? codes_bytes * 8 / packed_bits : max_slots_of(codec, codes_bytes);
     const Variant* var = packed_bits          ? variant_packed(codec)
                          : force_variant >= 0 ? variant_get(codec, force_variant)
-                                              : variant_get(codec, selected_variant(codec, max_slots, dict->width));
+                                              : variant_get(codec, column_variant(codec, max_slots, dict->width, n_strings));
     if (!var) return fail(FP_ERR_ARG, "no decode variant for codec %d", (int)codec);
     if (n_strings == 0xffffffffu) return fail(FP_ERR_ARG, "n_strings must be below 2^32-1");
     const uint64_t tile = variant_tile(*var);
@@ -336,7 +346,7 @@ fp_status run_rows(fp_codec codec, const fp_dict* dict, const void* d_codes, uin
     if (slots > 0xffffffffull) return fail(FP_ERR_ARG, "selected_slots %llu: at most 2^32-1", (unsigned long long)slots);
     const RowsLayout RL = rows_layout(codec, n_rows, slots);
     const uint64_t dec_slots = max_slots_of(codec, RL.codes_bytes);
-    const Variant* var = variant_get(codec, selected_variant(codec, dec_slots, dict->width));
+    const Variant* var = variant_get(codec, column_variant(codec, dec_slots, dict->width, n_rows));
     if (!var) return fail(FP_ERR_ARG, "no decode variant for codec %d", (int)codec);
     int per_wave = 0, sms = 0;
     fp_status st = grid_for(*var, &per_wave, &sms);

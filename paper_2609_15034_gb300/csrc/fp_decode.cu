@@ -61,11 +61,23 @@ const Variant* variant_get(int codec, int v) {
 // 16); the dictionary's width picks between them.
 //
 // Below 2^17 slots (256 tiles of 512: one to a warp of 16 blocks) the whole
-// column goes to one cluster in one launch: 8.7-9.5 us a call back to back
-// against 12.5-13.4 for three launches, alone 24-26 against 27-29, for every
-// codec from 1k to 88k slots; at 146k-177k slots the cluster's 16 SMs are
-// the slower side (13.3-17.6 us against 12.8-13.4).  Split-read dictionaries
-// keep the three launches.
+// column goes to one cluster in one launch: 9.0-10.0 us a call back to back
+// against 13.0-14.6 for three launches, alone 23.8-27.7 against 26.7-29.1, from
+// 9k to 125k slots (OnPair-16, whose tiles have half the slots, 12.8-14.0
+// against 13.2-13.7 from 80k on, alone 29.6-30.4 against 29.1); at 146k-177k
+// slots the cluster's 16 SMs are the slower side (13.3-17.6 us against
+// 12.8-13.4).  Four host-launched streams: 4.8 us a call, one launch's host time,
+// against 8.1; four streams of graphs, 18k slots: 1.8-2.1 against 2.4-3.0.  What
+// it costs is throughput with the GPU full of small columns: 16 streams of
+// graphs, 1.0-1.1 us against 0.73-0.86 at 18k slots, 1.2-1.8 against 0.8-1.05
+// at 100k.  Split-read dictionaries keep the three launches.
+//
+// A cluster's 256 warps also write every string's offset: with 2^17 strings
+// or more the three launches are the faster side
+// (100k slots: 100k strings 13.6-18.7 us against 14.5-15.7, 300k strings
+// 22.6-30.6 against 18.9-26.2, 4M strings 189-299 against 119-239).
+uint64_t cluster_strings_limit() { return 1ull << 17; }
+
 int variant_default(int codec, uint64_t max_slots, int width) {
     const bool split = width != 16;
     if (max_slots < (1ull << 17)) {

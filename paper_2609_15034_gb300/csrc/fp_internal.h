@@ -162,6 +162,8 @@ const Variant* variant_get(int codec, int v);
 // Default for a code buffer of max_slots slots and a dictionary read width
 // (8 or 16; only the OnPair codecs have both).
 int variant_default(int codec, uint64_t max_slots, int width);
+// Strings from which on a column does not take the one-cluster decode by default.
+uint64_t cluster_strings_limit();
 // The decoder of codes bit-packed at a run-time width (fp_decode_packed):
 // one warp-tile variant per escape-free codec, null for FSST-8.
 const Variant* variant_packed(int codec);
