@@ -55,10 +55,13 @@ const Variant* variant_get(int codec, int v) {
 // with the table read through L1; OnPair-16, 2M strings, 174 against 198 for
 // blocks of 8 warps; FSST-8, 16M strings, 529 with 32-slot lanes against 562
 // for blocks of 8 warps and 698 with 16-slot lanes; FSST-12, 20k documents, 99
-// with 32-slot lanes, 106 with 16, 130 through L1.  The smaller shapes below
-// 2^23 and 2^22 slots are the built-in rule where no tuned one is loaded.  The
-// OnPair codecs come in both read widths (split read W = 8, whole entries W =
-// 16); the dictionary's width picks between them.
+// with 32-slot lanes, 106 with 16, 130 through L1.  This is the rule where no
+// tuned shape is loaded.  OnPair-12 stages its table at every size (calls of
+// 2^17 .. 2^23 slots, staged against through L1: 11.9 : 14.0, 12.0 : 14.5, 12.0 :
+// 15.7, 17.0 : 17.2, 22.5 : 25.4, 30.9 : 39.4, 52.3 : 67.6 us; split reads 11.9 :
+// 14.9 .. 51.9 : 73.6); FSST-8 and FSST-12 take 16-slot lanes below 2^22 and 2^23
+// slots.  The OnPair codecs come in both read widths (split read W = 8, whole
+// entries W = 16); the dictionary's width picks between them.
 //
 // Below 2^17 slots (256 tiles of 512: one to a warp of 16 blocks) the whole
 // column goes to one cluster in one launch: 9.0-10.0 us a call back to back
@@ -73,9 +76,9 @@ const Variant* variant_get(int codec, int v) {
 // at 100k.  Split-read dictionaries keep the three launches.
 //
 // A cluster's 256 warps also write every string's offset: with 2^17 strings
-// or more the three launches are the faster side
-// (100k slots: 100k strings 13.6-18.7 us against 14.5-15.7, 300k strings
-// 22.6-30.6 against 18.9-26.2, 4M strings 189-299 against 119-239).
+// or more the three launches are the faster side (100k slots: 100k strings
+// 13.6-18.7 us against 14.5-15.7, 300k strings 22.6-30.6 against 18.9-26.2, 4M
+// strings 189-299 against 119-239).
 uint64_t cluster_strings_limit() { return 1ull << 17; }
 
 int variant_default(int codec, uint64_t max_slots, int width) {
@@ -91,8 +94,7 @@ int variant_default(int codec, uint64_t max_slots, int width) {
     }
     switch (codec) {
         case FP_ONPAIR12:
-            if (max_slots >= (1ull << 23)) return split ? 6 : 8;
-            return split ? 9 : 7;
+            return split ? 6 : 8;
         case FP_ONPAIR16: return split ? 5 : 4;
         case FP_FSST8: return max_slots >= (1ull << 22) ? 4 : 2;
         case FP_FSST12: return max_slots >= (1ull << 23) ? 2 : 0;
