@@ -486,7 +486,7 @@ typedef struct fp_serve_stats_t {
     uint64_t dict_hits, dict_misses, dict_evictions, dicts_registered;
     uint64_t inflight_bytes, peak_inflight_bytes;
     uint32_t inflight_requests;
-    uint32_t reserved;
+    uint32_t staged_waves;            /* waves decoded by the staged configuration       */
 } fp_serve_stats_t;
 
 /* Create a server on the current device (allocates the output arena and the

@@ -183,7 +183,7 @@ class ServeStats(ctypes.Structure):
                 ("dict_hits", ctypes.c_uint64), ("dict_misses", ctypes.c_uint64), ("dict_evictions", ctypes.c_uint64),
                 ("dicts_registered", ctypes.c_uint64), ("inflight_bytes", ctypes.c_uint64),
                 ("peak_inflight_bytes", ctypes.c_uint64), ("inflight_requests", ctypes.c_uint32),
-                ("reserved", ctypes.c_uint32)]
+                ("staged_waves", ctypes.c_uint32)]
 
 
 class Dict:

@@ -324,6 +324,9 @@ void lane_launch(fp_server* S, Lane& L) {
     }
     L.busy = true;
     S->st.waves++;
+    uint32_t kind = 0;
+    fp_batch_config_info(config, nullptr, nullptr, &kind);
+    if (kind == 2) S->st.staged_waves++;
     if (L.reqs.size() > S->st.max_wave_seen) S->st.max_wave_seen = (uint32_t)L.reqs.size();
 }
 
