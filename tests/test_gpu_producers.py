@@ -29,6 +29,13 @@ def fp():
     return m
 
 
+@pytest.fixture(scope="module")
+def streams(fp):
+    """Two streams for the whole file (torch hands out 32 and then the first again)."""
+    import torch
+    return torch.cuda.Stream(), torch.cuda.Stream()
+
+
 def device(a):
     import torch
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
@@ -73,7 +80,7 @@ class Pair:
 
 @pytest.mark.parametrize("codec", CODECS)
 @pytest.mark.parametrize("n", SIZES)
-def test_rows_right_after_their_producer(fp, codec, n):
+def test_rows_right_after_their_producer(fp, streams, codec, n):
     import torch
     cols = columns(codec, n)
     ids = [np.random.default_rng(s).integers(0, n, n // 2).astype(np.uint32) for s in (1, 2)]
@@ -81,7 +88,7 @@ def test_rows_right_after_their_producer(fp, codec, n):
             for c, i in zip(cols, ids)]
     x = Pair(fp, cols, [c.stream for c in cols], refs, ids)
     slots = max(int((c.code_offsets[i + 1] - c.code_offsets[i]).sum()) for c, i in zip(cols, ids))
-    s = torch.cuda.Stream()
+    s = streams[0]
     with torch.cuda.stream(s):
         for k in range(60):
             x.produce(k)
@@ -96,7 +103,7 @@ def test_rows_right_after_their_producer(fp, codec, n):
 @pytest.mark.parametrize("codec,bits", [(synth.ONPAIR16, 13), (synth.ONPAIR12, 11), (synth.FSST12, 10),
                                         (synth.FSST12, 9)])
 @pytest.mark.parametrize("n", SIZES)
-def test_packed_right_after_its_producer(fp, codec, bits, n):
+def test_packed_right_after_its_producer(fp, streams, codec, bits, n):
     import torch
     cols = columns(codec, n)
     rng = np.random.default_rng(bits)
@@ -105,7 +112,7 @@ def test_packed_right_after_its_producer(fp, codec, bits, n):
     refs = [oracle.decode_packed(codec, bits, c.dictionary.data, c.dictionary.offsets, st, c.code_offsets)
             for c, st in zip(cols, streams)]
     x = Pair(fp, cols, streams, refs)
-    s = torch.cuda.Stream()
+    s = streams[0]
     with torch.cuda.stream(s):
         for k in range(60):
             x.produce(k)
@@ -125,13 +132,13 @@ def call(fp, x, codec, n, stream):
 
 @pytest.mark.parametrize("codec", CODECS)
 @pytest.mark.parametrize("n", SIZES)
-def test_decode_behind_an_event(fp, codec, n):
+def test_decode_behind_an_event(fp, streams, codec, n):
     """The column is written on another stream, whose event the call's stream
     waits for, with the call before it still on the stream."""
     import torch
     cols = columns(codec, n)
     x = Pair(fp, cols, [c.stream for c in cols], [oracle_decode(c) for c in cols])
-    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    a, b = streams
     for k in range(30):
         a.wait_stream(b)
         with torch.cuda.stream(a):
