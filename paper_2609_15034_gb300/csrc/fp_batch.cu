@@ -581,10 +581,12 @@ struct fp_plan {
 namespace {
 
 // Host image of a batch's device tables.  The device layout is
-//   chunk records (per queue) | ticket -> chunk (per queue) | index blocks |
-//   tile -> first string (per chunk) | look-back words (per tile);
-// the image holds the first three parts (`table_bytes`); the index pass
-// writes the fourth and the look-back words are tagged per launch.
+//   chunk records (per queue) | ticket -> chunk, or units where the
+//   configuration is staged (per queue) | index blocks | tile-scan blocks |
+//   tile -> first string (per chunk) | look-back words (per tile) |
+//   tile elements | scanned tile offsets;
+// the image holds the tables in front of the first strings (`table_bytes`);
+// the index pass writes these, and the look-back words are tagged per launch.
 struct LayoutImage {
     std::vector<char> bytes;
     size_t o_src[kQueues], o_tc[kQueues], o_un[kQueues], o_ib, o_sb, o_first, o_ts, o_agg, o_ex, table_bytes, total_bytes;
@@ -661,8 +663,9 @@ fp_status make_layout(const fp_chunk* chunks, uint32_t n, const BatchKernel& BK,
             for (uint64_t b = 0; b < n_sb; ++b) sblk.push_back(make_uint2(((uint32_t)q << 30) | ci, (uint32_t)b));
             sb_glob += n_sb;
             src[q].push_back(s);
-            tchunk[q].insert(tchunk[q].end(), nt, ci);
-            if (BK.unit[q]) {
+            if (!BK.unit[q]) {
+                tchunk[q].insert(tchunk[q].end(), nt, ci);
+            } else {
                 const uint64_t nu = (nt + unit_tiles - 1) / unit_tiles;   // equal parts
                 for (uint64_t u = 0; u < nu; ++u) {
                     const uint64_t t0 = nt * u / nu, t1 = nt * (u + 1) / nu;

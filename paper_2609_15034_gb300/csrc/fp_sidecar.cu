@@ -59,12 +59,12 @@ __global__ void __launch_bounds__(32) sidecar_check_kernel(const u64* total, u64
 
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Scratch: workspace header | look-back words of the tile scan | extent |
-// tile elements | tile -> first string.
+// Scratch: workspace header | look-back words of the tile scan | tile elements |
+// tile -> first string.
 struct Layout {
     uint64_t n_tiles;   // upper bound on the column's tiles
     uint64_t n_scan;
-    size_t o_status, o_extent, o_agg, o_first, bytes;
+    size_t o_status, o_agg, o_first, bytes;
 };
 
 Layout layout(int codec, uint64_t codes_bytes) {
@@ -72,8 +72,7 @@ Layout layout(int codec, uint64_t codes_bytes) {
     L.n_tiles = max_slots_of(codec, codes_bytes) / tile_slots(codec) + 2;
     L.n_scan = L.n_tiles / kScanTile + 2;
     L.o_status = al256(kWsHeaderBytes);
-    L.o_extent = L.o_status + al256(L.n_scan * sizeof(u64));
-    L.o_agg = L.o_extent + al256(sizeof(Extent));
+    L.o_agg = L.o_status + al256(L.n_scan * sizeof(u64));
     L.o_first = L.o_agg + al256(L.n_tiles * sizeof(u64));
     L.bytes = L.o_first + al256((L.n_tiles + 1) * sizeof(u32));
     return L;
