@@ -108,10 +108,10 @@ def test_packed_right_after_its_producer(fp, streams, codec, bits, n):
     cols = columns(codec, n)
     rng = np.random.default_rng(bits)
     codes_of = [rng.integers(0, 200, c.n_slots).astype(np.uint32) for c in cols]
-    streams = [pack_bits(c, bits) for c in codes_of]
+    packed = [pack_bits(c, bits) for c in codes_of]
     refs = [oracle.decode_packed(codec, bits, c.dictionary.data, c.dictionary.offsets, st, c.code_offsets)
-            for c, st in zip(cols, streams)]
-    x = Pair(fp, cols, streams, refs)
+            for c, st in zip(cols, packed)]
+    x = Pair(fp, cols, packed, refs)
     s = streams[0]
     with torch.cuda.stream(s):
         for k in range(60):
