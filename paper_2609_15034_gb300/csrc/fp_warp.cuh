@@ -806,9 +806,11 @@ struct WarpCore {
     // the kernel that writes the column ended).
     static __device__ __forceinline__ void strings_begin(const DecodeParams& p, u32 lo, u32 hi, Strings& sb) {
         const u32 nb_col = p.n_strings + 1u;
+        const u32 lane = threadIdx.x & 31u;
+        lo = min(lo, nb_col);
         hi = min(hi, nb_col);
-        sb.first = min(lo, nb_col) + (threadIdx.x & 31u);
-        sb.left = sb.first < hi ? hi - sb.first : 0u;
+        sb.first = lo + lane;   // (may pass 2^32 where nothing is left)
+        sb.left = hi > lo && hi - lo > lane ? hi - lo - lane : 0u;
 #pragma unroll
         for (int j = 0; j < PB; ++j) sb.pos[j] = 32u * j < sb.left ? in_order(p.code_offsets + sb.first + 32u * j) : 0u;
     }
