@@ -439,11 +439,13 @@ fp_status fp_dict_upload(fp_codec codec, const uint8_t* h_bytes, const uint32_t*
     d->n_entries = n_entries;
     d->table_bytes = table.size();
     // OnPair: the two 8-byte planes of the entries (for split reads) and the
-    // read width.  The default is 16: on GB300 this decoder read whole
-    // entries faster than split reads for every share of long tokens from 0
-    // to 100 % (1-3 % with the table in shared memory, 5-13 % through L1), so
-    // the paper's rule (fp_width_for_histogram) is left to callers, through
-    // fp_dict_set_width.
+    // read width.  The default is 16: whole entries are the faster side or
+    // within 4 % of it at every share of long tokens (36M codes, uniform and
+    // Zipf: OnPair-12 0-3 % faster up to 75 % long, 6 % at 100 %; OnPair-16 2-13 %
+    // faster at 25 % long, 10-42 % from 50 % on; with no long token at all split
+    // reads are 1-3 % faster for OnPair-16, and 2 % for OnPair-12 at 3M codes),
+    // so the paper's rule (fp_width_for_histogram) is left to callers,
+    // through fp_dict_set_width.
     std::vector<uint8_t> planes;
     d->width = is_onpair(codec) ? 16 : 8;
     if (is_onpair(codec)) {
