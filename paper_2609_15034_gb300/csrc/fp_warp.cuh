@@ -53,7 +53,7 @@ __device__ __forceinline__ Elem wt_unpack(u64 w) {
 // selects per word and at most two stores, one for FSST symbols.  The decode
 // kernel, 16-byte window -> 32-bit -> 64-bit words: OnPair-12, 36M codes 149 ->
 // 118 -> 110 us; FSST-8, 38M slots 134 -> 93 -> 92; FSST-12, 33M codes 110 -> 72
-// -> 70.  What bounds it now is the shared-memory pipe (84 % of its wavefronts
+// -> 70.  What bounds it now is the shared-memory pipe (77 % of its wavefronts
 // on OnPair-12: about 10 per 32 codes for the table reads, 8 for these
 // stores, 3 for the lengths), with the ALU pipe at 66 %.
 struct StageWriter {
