@@ -174,18 +174,21 @@ __device__ __forceinline__ u32 bits_below(int b) { return b <= 0 ? 0u : (b >= 32
 // the stored stream shifted into place, where a byte or two per slot took up
 // to 16 loads and a search over all rows 20 more.
 //
-// The window holds a chunk of one-code rows, so that every lane finds its rows
-// in the first one; with one of 64 rows the lanes past it searched global
-// memory row by row.  500k of 5M rows, a whole call, a byte or two per slot ->
-// window of 64 -> this: OnPair-12, 1 code a row 61.6 -> 73.9 -> 48.1 us, 2 codes
-// 58.0 -> 59.5 -> 37.9, 18 codes 122.9 -> 88.7 -> 90.2; FSST-8 64.3 -> 121.6 ->
-// 57.0, 63.8 -> 85.5 -> 45.6, 141.8 -> 81.6 -> 82.7.  A chunk of more rows than
-// kRowWindows windows hold (almost all of them empty) has the rest searched in
-// global memory.  Slots past the selected total (or the bound) are not written
-// and never decoded.
-constexpr u32 kRowWindows = 8;
-// Blocks per SM: FSST-8's window of 512 rows takes 32 KiB a block; with six
-// blocks L1 is left too little (18 codes a row: 103.5 us against 82.7).
+// The window holds a chunk of one-code rows (half of one of FSST-8's), so that
+// nearly every lane finds its rows in the first one; with one of 64 rows the
+// lanes past it searched global memory row by row.  500k of 5M rows, a whole
+// call, a byte or two per slot -> window of 64 -> this: OnPair-12, 1 code a row
+// 62.1 -> 74.0 -> 45.1 us, 2 codes 58.0 -> 59.6 -> 37.4, 18 codes 123.4 -> 88.8 ->
+// 89.4; FSST-8 65.0 -> 121.8 -> 60.8, 64.2 -> 85.2 -> 47.2, 141.2 -> 81.4 -> 80.6.
+// (FSST-8 with 512 rows: 1 code 57.0, but 20M selected slots of 13 codes a row
+// 136 against 129: the window takes the L1 that the words need.)  A chunk of
+// more rows than kRowWindows windows hold (almost all of them empty) has the
+// rest searched in global memory.  Slots past the selected total (or the
+// bound) are not written and never decoded.
+constexpr u32 kRowWindow = 256, kRowWindows = 8;
+// Blocks per SM that the registers allow without spilling (48 for FSST-8's
+// groups of 16 slots, else 40; 8 blocks of 32 registers spill and are 2-8 %
+// slower per call).
 __host__ __device__ constexpr int row_gather_blocks(int codec) { return codec == FP_FSST8 ? 5 : 6; }
 
 template <int CODEC>
@@ -194,7 +197,7 @@ __global__ void __launch_bounds__(kRowBlock, row_gather_blocks(CODEC)) rows_gath
                                                               const WsHeader* ws) {
     constexpr int BITS = CODEC == FP_ONPAIR16 ? 16 : (CODEC == FP_FSST8 ? 8 : 12);
     constexpr int G = CODEC == FP_FSST8 ? 16 : 8, CH = 32 * G, NW = G * BITS / 32;
-    constexpr u32 WIN = CODEC == FP_FSST8 ? 512 : 256;
+    constexpr u32 WIN = kRowWindow;
     __shared__ u32 s_v[kRowBlock / 32][WIN + 1], s_src[kRowBlock / 32][WIN];
     grid_wait();
     grid_release();
@@ -233,9 +236,15 @@ __global__ void __launch_bounds__(kRowBlock, row_gather_blocks(CODEC)) rows_gath
             const long long bit = (long long)BITS * ((long long)sb + v0 - vs);
             const u32 w0 = (u32)(bit >> 5);
             const u32 q_lo = j * BITS / 32u, q_hi = (end * BITS - 1u) / 32u + 1u;
+            // one check for all of them: a check per word cost 3 % of a call
             u32 x[NW + 1];
+            if (bit >= 0 && (u64)w0 + NW < n_words) {
 #pragma unroll
-            for (int q = 0; q <= NW; ++q) x[q] = (u32)q >= q_lo && (u32)q <= q_hi ? word(w0 + q) : 0u;
+                for (int q = 0; q <= NW; ++q) x[q] = (u32)q >= q_lo && (u32)q <= q_hi ? __ldg(words + w0 + q) : 0u;
+            } else {
+#pragma unroll
+                for (int q = 0; q <= NW; ++q) x[q] = word(w0 + q);
+            }
 #pragma unroll
             for (int q = 0; q < NW; ++q) {
                 const u32 keep = j ? bits_below((int)j * BITS - 32 * q) : 0u;
